@@ -704,15 +704,16 @@ __global__ void k_long_direct(const __grid_constant__ LongArgs la, int q) {
 // Approximate top-k of the products x_i y_j (Alg. 9 with the NormQueue), for
 // `batch` independent pairs of length n (2n - 1 <= 8192), each run twice (y,
 // and y reversed for the index recovery):
-//   k_topk_sums  one CTA per (problem, direction): the p-sums of every p of P
-//                for every diagonal m = i + j (the FFT level above), and the
-//                first estimate psi_m;
-//   k_topk_pop   one warp per (problem, direction): k NormQueue pops -- the
-//                diagonal with the largest psi (two-level argmax over blocks
-//                of 32 diagonals), its value, the subtraction of psi^p from
-//                every p-sum of that diagonal, the re-estimate clamped to the
-//                value just popped; a diagonal is exhausted after as many
-//                pops as it has terms;
+//   k_topk_sums  the p-sums of every p of P for every diagonal m = i + j (one
+//                FFT convolution per problem, direction and p);
+//   k_topk_merge k <= TOPK_KMAX NormQueue pops, every diagonal's at once: a pop
+//                takes the diagonal with the largest estimate psi, subtracts
+//                psi^p from every p-sum of that diagonal and re-estimates,
+//                clamped to the value just popped; a diagonal is exhausted
+//                after as many pops as it has terms;
+//   k_topk_first, k_topk_pop  the same pops for larger k, one after another
+//                (one warp per problem and direction, a two-level argmax over
+//                blocks of 32 diagonals);
 //   k_topk_index i = (m1 + m2 - n + 1) / 2, j = m1 - i from the diagonals of
 //                the two calls' pops of equal rank, kept when x_i y_j agrees
 //                with the popped value within TOPK_VERIFY.
@@ -729,7 +730,7 @@ struct TopkArgs {
   double* psi0;    // [batch][2][nz] estimates (the first, then kept by the pops)
   double* bmax0;   // [batch][2][nb] the largest estimate of each block of 32 diagonals
   uint16_t* left;  // [batch][2][nz] terms of each diagonal not yet popped
-  double* scale;   // [batch] max x * max y
+  double* scale;   // [batch] max x * max y, -1 where the input is out of the domain
   int32_t* diag;   // [batch][2][k]
   float* vals;     // [batch][ldk]
   int32_t* out_i;
@@ -764,73 +765,296 @@ __device__ __forceinline__ double pow_pow2(double a, int plog) {
   return a;
 }
 
+// ---- transforms of the p-sums.  The same radix-2 butterflies, twiddles and
+// operation order as fft_dit / conv_level (every p-sum has the same bits),
+// but eight values per thread stay in registers for three stages, so a
+// transform of 2^13 makes 9 passes over shared memory with a barrier each
+// instead of 28, and nothing is permuted: the forward transform reads natural
+// order and leaves frequency k at address bitrev(k); the last forward stage
+// pairs the addresses of k and k + N/2, which the spectrum needs together
+// with those of N - k and N/2 - k, so it is fused into the spectrum; the
+// spectrum's half-length sequence, left in the even addresses in
+// bit-reversed order, is what the decimation in time starts from.
+// What bounds it is the FP64 issue rate (two lanes per clock and SM): about
+// 6.8e5 FP64 instructions per level at N = 2^13.
+
+// Shared-memory slot of element i: bits 1-2 are XORed with bits 4-5, so that
+// the passes with a stride of two or eight elements spread over the banks.
+__device__ __forceinline__ int slot(int i) { return i ^ (((i >> 4) & 3) << 1); }
+
+__device__ __forceinline__ void bfly(double2& u, double2& v, double2 t) {
+  const double2 a = u;
+  u = make_double2(a.x + t.x, a.y + t.y);
+  v = make_double2(a.x - t.x, a.y - t.y);
+}
+
+// R stages s .. s + R - 1 of a transform of 2^lg values on the 2^R values
+// v[r] of one group; v[r] sits at position j + (r << s) within its block of
+// 2^(s + R) (positions as in fft_dit).  tw[k << tsh] = exp(-2 pi i k / 2^lg).
+template <int R, bool INV>
+__device__ __forceinline__ void group_stages(double2 (&v)[1 << R], const double2* tw, int lg,
+                                             int tsh, int s, int j) {
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+    const int sh = lg - 1 - s - t + tsh;
+#pragma unroll
+    for (int o = 0; o < (1 << t); ++o) {
+      const double2 w = tw[(j + (o << s)) << sh];
+#pragma unroll
+      for (int r = 0; r < (1 << R); r += 2 << t) {
+        const double2 b = v[r + o + (1 << t)];
+        bfly(v[r + o], v[r + o + (1 << t)], INV ? cmulc(w, b) : cmul(w, b));
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ int rev_bits(int k, int n) {
+  return n == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - n));
+}
+
+// Forward stages s .. s + R - 1 in place: the address of a position is its bit
+// reversal, so stage t pairs addresses that differ in bit lg - 1 - t.
+template <int R>
+__device__ __forceinline__ void fwd_pass(double2* a, const double2* tw, int lg, int s) {
+  const int low = lg - s - R;  // address bits below the group's
+  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+    const int hi = g >> low, base = (hi << (low + R)) | (g & ((1 << low) - 1));
+    double2 v[1 << R];
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(base + (rev_bits(r, R) << low))];
+    group_stages<R, false>(v, tw, lg, 0, s, rev_bits(hi, s));
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) a[slot(base + (rev_bits(r, R) << low))] = v[r];
+  }
+  __syncthreads();
+}
+
+// Inverse stages s .. s + R - 1 of the 2^lg values in the even addresses.
+template <int R>
+__device__ __forceinline__ void inv_pass(double2* a, const double2* tw, int lg, int s) {
+  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+    const int j = g & ((1 << s) - 1), base = ((g >> s) << (s + R)) | j;
+    double2 v[1 << R];
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(2 * (base + (r << s)))];
+    group_stages<R, true>(v, tw, lg, 1, s, j);
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) a[slot(2 * (base + (r << s)))] = v[r];
+  }
+  __syncthreads();
+}
+
+// First forward pass of R = 3 stages straight from the powered values: group j
+// holds the addresses j + t N / 8, of which t >= 4 are zero (n <= N / 2), so
+// stage 0 copies, stage 1 multiplies by 1 and -i, and half of stage 2 does.
+__device__ __forceinline__ void first_pass8(double2* a, const double2* tw, int lg, int j,
+                                            const double (&x)[4], const double (&y)[4]) {
+  double2 v[8];
+#pragma unroll
+  for (int r = 0; r < 8; r += 2) {
+    const int t = ((r >> 1) & 1) * 2 + (r >> 2);  // rev3(r), r even
+    v[r] = v[r + 1] = make_double2(x[t], y[t]);
+  }
+#pragma unroll
+  for (int r = 0; r < 8; r += 4) {
+    bfly(v[r], v[r + 2], v[r + 2]);
+    bfly(v[r + 1], v[r + 3], make_double2(v[r + 3].y, -v[r + 3].x));
+  }
+  bfly(v[0], v[4], v[4]);
+  bfly(v[1], v[5], cmul(tw[1 << (lg - 3)], v[5]));
+  bfly(v[2], v[6], make_double2(v[6].y, -v[6].x));
+  bfly(v[3], v[7], cmul(tw[3 << (lg - 3)], v[7]));
+#pragma unroll
+  for (int r = 0; r < 8; ++r) a[slot(j + (rev_bits(r, 3) << (lg - 3)))] = v[r];
+}
+
+// The spectrum from the packed pair's transform (all but its last stage done)
+// to the half-length sequence 8 V_k in the even addresses; see conv_level.
+// The halves of the formulas there are left out: a power of two, exact.
+__device__ __forceinline__ void spectrum_pass(double2* a, const double2* tw, int lg) {
+  const int lm = lg - 1, M = 1 << lm;
+  for (int e = threadIdx.x; e <= (M >> 1); e += blockDim.x) {
+    // p = bitrev(k): 0, then the lower half of every [2^h, 2^(h + 1)); the
+    // address of M - k mirrors p within that range
+    int p = e, pm = e;
+    if (e > 1) {
+      const int f = e - 1, hb = 1 << (31 - __clz(f));
+      p = f + hb;
+      pm = p ^ (2 * hb - 1);
+    }
+    if (e > M >> 1 || p >= M) continue;
+    const int k = rev_bits(p, lm);
+    double2 ak = a[slot(2 * p)], amk = a[slot(2 * p + 1)];  // frequencies k, k + M
+    bfly(ak, amk, cmul(tw[k], amk));
+    double2 am = ak, an = amk;                              // M - k, N - k
+    if (k == 0) {
+      an = ak;  // N - 0 = 0 and M - 0 = M
+      am = amk;
+    } else if (pm != p) {
+      am = a[slot(2 * pm)];
+      an = a[slot(2 * pm + 1)];
+      bfly(am, an, cmul(tw[M - k], an));
+    }
+    auto z4 = [](double2 u, double2 v) {  // 4 spec_z
+      return cmul(make_double2(u.x + v.x, u.y - v.y), make_double2(u.y + v.y, -(u.x - v.x)));
+    };
+    auto v8 = [](double2 zk, double2 zm, double2 w) {  // 8 spec_v
+      const double2 o = cmulc(w, make_double2(zk.x - zm.x, zk.y + zm.y));
+      return make_double2((zk.x + zm.x) - o.y, (zk.y - zm.y) + o.x);
+    };
+    const double2 zk = z4(ak, an), zm = z4(am, amk);
+    a[slot(2 * p)] = v8(zk, zm, tw[k]);
+    if (k != 0 && pm != p) a[slot(2 * pm)] = v8(zm, zk, tw[M - k]);
+  }
+  __syncthreads();
+}
+
+// The p-sums.  Work items (problem, direction, level) in this order, each CTA
+// a contiguous run of them: the items spread over all SMs (one CTA per
+// problem and direction ran 512 pairs of the 256-problem batch as 3.37 waves
+// of 152, the last one mostly empty), and the values x'^p, y'^p of a pair stay
+// in registers and are squared from level to level.
+// 256 problems of n = 4096, 13 levels: 8.24 ms (12.29 ms with one CTA per
+// problem and direction and two stages per pass).
 __global__ void __launch_bounds__(FFT_THREADS, 1)
     k_topk_sums(const __grid_constant__ TopkArgs ta) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N = 1 << ta.logN;
+  const int lg = ta.logN, N = 1 << lg;
   double2* a = reinterpret_cast<double2*>(smem);
   double2* tw = a + N;
   __shared__ float red[2][FFT_THREADS / 32];
-  const int b = blockIdx.x >> 1, dir = blockIdx.x & 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* x = ta.x + (int64_t)b * ta.ldx;
-  const float* y = ta.y + (int64_t)b * ta.ldy;
-  for (int k = tid; k < (N >> 1); k += FFT_THREADS) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - ta.logN)];
-  float mx = 0.0f, my = 0.0f;
-  bool bad = false;
-  for (int k = tid; k < ta.n; k += FFT_THREADS) {
-    const float u = x[k], v = y[k];
-    bad |= !(u >= 0.0f && u <= 3.4028235e38f) || !(v >= 0.0f && v <= 3.4028235e38f);
-    mx = fmaxf(mx, u);
-    my = fmaxf(my, v);
-  }
-  if (__syncthreads_or(bad)) {
-    if (tid == 0) set_status(ta.status, PN_EDOMAIN);
-    return;
-  }
+  const int nt = static_cast<int>(blockDim.x), nw = nt >> 5;
+  for (int k = tid; k < (N >> 1); k += nt) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - lg)];
+  const int64_t items = (int64_t)2 * ta.batch * ta.n_p;
+  const int64_t first = items * blockIdx.x / gridDim.x, last = items * (blockIdx.x + 1) / gridDim.x;
+  const int groups = N >> 3;  // of the first pass (N >= 8)
+  double xv[2][4], yv[2][4];  // the thread's values of the current pair (N >= 8)
+  double sx = 1.0, sy = 1.0;
+  int plog = 0;
+  bool skip = false;          // the pair's input is out of the domain
+  for (int64_t it = first; it < last; ++it) {
+    const int pd = static_cast<int>(it / ta.n_p), q = static_cast<int>(it - (int64_t)pd * ta.n_p);
+    const int b = pd >> 1, dir = pd & 1;
+    const float* x = ta.x + (int64_t)b * ta.ldx;
+    const float* y = ta.y + (int64_t)b * ta.ldy;
+    if (it == first || q == 0) {
+      float mx = 0.0f, my = 0.0f;
+      bool bad = false;
+      for (int k = tid; k < ta.n; k += nt) {
+        const float u = x[k], v = y[k];
+        bad |= !(u >= 0.0f && u <= 3.4028235e38f) || !(v >= 0.0f && v <= 3.4028235e38f);
+        mx = fmaxf(mx, u);
+        my = fmaxf(my, v);
+      }
+      skip = __syncthreads_or(bad);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, off));
-  }
-  if (lane == 0) {
-    red[0][warp] = mx;
-    red[1][warp] = my;
-  }
-  __syncthreads();
-  double sx = 0.0, sy = 0.0;
-  for (int w = 0; w < FFT_THREADS / 32; ++w) {
-    sx = fmax(sx, static_cast<double>(red[0][w]));
-    sy = fmax(sy, static_cast<double>(red[1][w]));
-  }
-  if (sx == 0.0) sx = 1.0;
-  if (sy == 0.0) sy = 1.0;
-  if (tid == 0 && dir == 0) ta.scale[b] = sx * sy;
-  MaxconvArgs ma;
-  ma.nx = ta.n;
-  ma.ny = ta.n;
-  ma.logN = ta.logN;
-  const double invM = 2.0 / N;
-  double* sig = ta.sig + (int64_t)blockIdx.x * ta.n_p * ta.nz;
-  for (int q = 0; q < ta.n_p; ++q) {
-    conv_level<true>(a, tw, ma, x, y, 1.0 / sx, 1.0 / sy, ta.p_log2[q], dir == 1);
-    for (int m = tid; m < ta.nz; m += FFT_THREADS)
-      sig[(int64_t)q * ta.nz + m] = ((m & 1) ? a[m >> 1].y : a[m >> 1].x) * invM;
-    __syncthreads();
-  }
-  // first estimates: the largest p with sigma >= tau (none: 0)
-  double* psi = ta.psi0 + (int64_t)blockIdx.x * ta.nz;
-  uint16_t* left = ta.left + (int64_t)blockIdx.x * ta.nz;
-  for (int m = tid; m < ta.nz; m += FFT_THREADS) {
-    double e = 0.0;
-    for (int q = ta.n_p - 1; q >= 0; --q) {
-      const double v = sig[(int64_t)q * ta.nz + m];
-      if (v >= ta.tau) {
-        e = root_fp64(v, ta.p_log2[q]);
-        break;
+      for (int off = 16; off > 0; off >>= 1) {
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, off));
+      }
+      if (lane == 0) {
+        red[0][warp] = mx;
+        red[1][warp] = my;
+      }
+      __syncthreads();
+      sx = sy = 0.0;
+      for (int w = 0; w < nw; ++w) {
+        sx = fmax(sx, static_cast<double>(red[0][w]));
+        sy = fmax(sy, static_cast<double>(red[1][w]));
+      }
+      if (sx == 0.0) sx = 1.0;
+      if (sy == 0.0) sy = 1.0;
+      if (tid == 0 && q == 0) {
+        if (skip) set_status(ta.status, PN_EDOMAIN);
+        if (dir == 0) ta.scale[b] = skip ? -1.0 : sx * sy;
+      }
+      plog = 0;
+      if (lg >= 3) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const int j = tid + u * nt, k = j + t * groups;
+            const bool in = j < groups && k < ta.n && !skip;
+            xv[u][t] = in ? static_cast<double>(x[k]) * (1.0 / sx) : 0.0;
+            yv[u][t] = in ? static_cast<double>(y[dir ? ta.n - 1 - k : k]) * (1.0 / sy) : 0.0;
+          }
       }
     }
-    psi[m] = e;
+    if (skip) continue;
+    if (lg >= 3) {
+      for (; plog < ta.p_log2[q]; ++plog) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            xv[u][t] = __dmul_rn(xv[u][t], xv[u][t]);
+            yv[u][t] = __dmul_rn(yv[u][t], yv[u][t]);
+          }
+      }
+    }
+    int s = 0;
+    if (lg >= 4) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (tid + u * nt < groups) first_pass8(a, tw, lg, tid + u * nt, xv[u], yv[u]);
+      s = 3;
+    } else {  // N <= 8: every stage below
+      for (int k = tid; k < N; k += nt) {
+        double u = 0.0, v = 0.0;
+        if (k < ta.n) {
+          u = static_cast<double>(x[k]) * (1.0 / sx);
+          v = static_cast<double>(y[dir ? ta.n - 1 - k : k]) * (1.0 / sy);
+          for (int t = 0; t < ta.p_log2[q]; ++t) {
+            u = __dmul_rn(u, u);
+            v = __dmul_rn(v, v);
+          }
+        }
+        a[slot(k)] = make_double2(u, v);
+      }
+    }
+    __syncthreads();
+    for (; s + 3 <= lg - 1; s += 3) fwd_pass<3>(a, tw, lg, s);
+    if (s + 2 == lg - 1) fwd_pass<2>(a, tw, lg, s);
+    else if (s + 1 == lg - 1) fwd_pass<1>(a, tw, lg, s);
+    spectrum_pass(a, tw, lg);
+    const int lm = lg - 1;
+    for (s = 0; s + 3 <= lm; s += 3) inv_pass<3>(a, tw, lm, s);
+    if (s + 2 == lm) inv_pass<2>(a, tw, lm, s);
+    else if (s + 1 == lm) inv_pass<1>(a, tw, lm, s);
+    const double scale = 0.25 / N;  // 2 / N, and the spectrum's 8
+    double* sig = ta.sig + ((int64_t)pd * ta.n_p + q) * ta.nz;
+    for (int m = tid; m < ta.nz; m += nt) {
+      const double2 v = a[slot(m & ~1)];
+      sig[m] = ((m & 1) ? v.y : v.x) * scale;
+    }
+    __syncthreads();
+  }
+}
+
+// First estimate psi_m: the largest p with sigma >= tau (none: 0).
+__device__ __forceinline__ int first_level(const TopkArgs& ta, const double* sig, int m, double& v) {
+  for (int q = ta.n_p - 1; q >= 0; --q) {
+    v = sig[(int64_t)q * ta.nz + m];
+    if (v >= ta.tau) return q;
+  }
+  return -1;
+}
+
+// First estimates, term counts and block maxima for k_topk_pop (large k).
+__global__ void __launch_bounds__(FFT_THREADS, 1)
+    k_topk_first(const __grid_constant__ TopkArgs ta) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double* sig = ta.sig + (int64_t)blockIdx.x * ta.n_p * ta.nz;
+  double* psi = ta.psi0 + (int64_t)blockIdx.x * ta.nz;
+  uint16_t* left = ta.left + (int64_t)blockIdx.x * ta.nz;
+  const bool ok = ta.scale[blockIdx.x >> 1] >= 0.0;  // else no p-sums were written: no pops
+  for (int m = tid; m < ta.nz; m += FFT_THREADS) {
+    double v = 0.0;
+    const int q = ok ? first_level(ta, sig, m, v) : -1;
+    psi[m] = q >= 0 ? root_fp64(v, ta.p_log2[q]) : 0.0;
     left[m] = static_cast<uint16_t>(terms_of(m, ta.n, ta.n));
   }
   __syncthreads();
@@ -843,6 +1067,212 @@ __global__ void __launch_bounds__(FFT_THREADS, 1)
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
     if (lane == 0) bmax[blk] = v;
+  }
+}
+
+// k NormQueue pops of one (problem, direction), k <= TOPK_KMAX, for all
+// diagonals at once.  A diagonal's pops depend on that diagonal alone: its
+// values alpha_1 = psi_m >= alpha_2 >= ... (each re-estimate is clamped to the
+// value popped before it), each from the diagonal's p-sums after the pops
+// before.  The queue always takes the largest value at hand, the smallest
+// diagonal among equals, so its k pops are the k first of all diagonals'
+// values in the order (value descending, diagonal ascending), and equal
+// pairs are interchangeable.  Hence: keep the k first values known so far;
+// a diagonal whose last known value is among them makes its next value (one
+// thread per diagonal); repeat until no last value is left among the k.  The
+// values are the sequential loop's bit for bit.
+// What bounds the sequential loop (k_topk_pop) is latency: 1024 dependent pops
+// of about 90 FP64 instructions of one warp, 64 cycles each at two FP64 lanes
+// per clock and SM.  Here a warp instruction serves 32 diagonals, and about
+// three rounds replace the 1024 steps.  256 problems of n = 4096, k = 1024:
+// 0.90 ms (6.34 ms with k_topk_pop).
+constexpr int TOPK_KMAX = 2048;
+constexpr int TOPK_THREADS = 256;
+
+// Values held at most: every diagonal at first, later k kept and as many new.
+__host__ __device__ inline int topk_cap(int nz, int k) {
+  int cap = 2;
+  while (cap < nz || cap < 2 * k) cap <<= 1;
+  return cap;
+}
+__host__ __device__ inline int topk_merge_smem(int nz, int k) {
+  return topk_cap(nz, k) * (8 + 2) + 2 * k;
+}
+
+// Sorts (val, dm) [0, count) by value descending, then diagonal ascending;
+// the arrays hold a power of two >= count entries.  Values are positive
+// doubles as their bits, which order alike, so that no compare takes the FP64
+// pipe.
+__device__ void topk_sort(uint64_t* val, uint16_t* dm, int count) {
+  int n2 = 2;
+  while (n2 < count) n2 <<= 1;
+  for (int i = count + threadIdx.x; i < n2; i += TOPK_THREADS) {
+    val[i] = 0u;
+    dm[i] = 0;
+  }
+  __syncthreads();
+  for (int size = 2; size <= n2; size <<= 1) {
+    for (int d = size >> 1; d > 0; d >>= 1) {
+      for (int e = threadIdx.x; e < (n2 >> 1); e += TOPK_THREADS) {
+        const int i = ((e & ~(d - 1)) << 1) | (e & (d - 1)), j = i + d;
+        const uint64_t vi = val[i], vj = val[j];
+        const uint16_t mi = dm[i], mj = dm[j];
+        const bool same = vi == vj;
+        const int di = mi & 0x1fff, dj = mj & 0x1fff;
+        if ((i & size) == 0 ? (vj > vi || (same && dj < di)) : (vi > vj || (same && di < dj))) {
+          val[i] = vj;
+          val[j] = vi;
+          dm[i] = mj;
+          dm[j] = mi;
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+__global__ void __launch_bounds__(TOPK_THREADS)
+    k_topk_merge(const __grid_constant__ TopkArgs ta) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr uint16_t TAIL = 0x2000;  // the last value made of its diagonal
+  const int cap = topk_cap(ta.nz, ta.k);
+  uint64_t* val = reinterpret_cast<uint64_t*>(smem);        // [cap] values, as bits
+  float* f = reinterpret_cast<float*>(smem);                // [nz], before val is used
+  uint16_t* dm = reinterpret_cast<uint16_t*>(val + cap);    // [cap] diagonal | TAIL
+  uint16_t* act = dm + cap;                                 // [k] entries to go on from
+  __shared__ int cnt, n_act;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int b = blockIdx.x >> 1, dir = blockIdx.x & 1;
+  double* sig = ta.sig + (int64_t)blockIdx.x * ta.n_p * ta.nz;
+  uint16_t* left = ta.left + (int64_t)blockIdx.x * ta.nz;
+  int32_t* diag = ta.diag + (int64_t)blockIdx.x * ta.k;
+  const double scale = ta.scale[b];
+  int kept = 0;
+  if (scale >= 0.0) {  // else: the input is out of the domain, no pops
+    // candidates: the first estimates to FP32 accuracy, and the diagonals at
+    // or above the k-th largest of them (less a margin far above FP32's error)
+    for (int m = tid; m < ta.nz; m += TOPK_THREADS) {
+      double v;
+      const int q = first_level(ta, sig, m, v);
+      float r = 0.0f;
+      if (q >= 0) {
+        r = static_cast<float>(v);
+        for (int s = 0; s < ta.p_log2[q]; ++s) r = sqrtf(r);
+        if (!(r > 0.0f)) r = static_cast<float>(root_fp64(v, ta.p_log2[q]));
+      }
+      f[m] = r;
+    }
+    if (tid == 0) cnt = 0;
+    __syncthreads();
+    // largest bit pattern T >= 1 that k values reach (1: fewer than k are positive)
+    uint32_t T = 1u;
+    if (ta.nz > ta.k) {
+      uint32_t lo = 1u, hi = 0x7f800001u;  // reached by >= k (or lo = 1), by < k
+      while (hi - lo > 1u) {
+        const uint32_t mid = lo + (hi - lo) / 2u;
+        int c = 0;
+        for (int m = tid; m < ta.nz; m += TOPK_THREADS) c += __float_as_uint(f[m]) >= mid;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0 && c) atomicAdd(&cnt, c);
+        __syncthreads();
+        const int total = cnt;
+        __syncthreads();
+        if (tid == 0) cnt = 0;
+        if (total >= ta.k) lo = mid;
+        else hi = mid;
+        __syncthreads();
+      }
+      T = lo;
+    }
+    const float thr = __uint_as_float(T) * (1.0f - 1e-5f);
+    for (int m0 = 0; m0 < ta.nz; m0 += TOPK_THREADS) {
+      const int m = m0 + tid;
+      const bool take = m < ta.nz && f[m] > 0.0f && f[m] >= thr;
+      const unsigned bal = __ballot_sync(0xffffffffu, take);
+      int at = 0;
+      if (lane == 0 && bal) at = atomicAdd(&cnt, __popc(bal));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (take) dm[at] = static_cast<uint16_t>(m);
+    }
+    __syncthreads();
+    int total = cnt;
+    for (int c = tid; c < total; c += TOPK_THREADS) {
+      const int m = dm[c];
+      double v;
+      const int q = first_level(ta, sig, m, v);
+      val[c] = __double_as_longlong(q >= 0 ? root_fp64(v, ta.p_log2[q]) : 0.0);
+      left[m] = static_cast<uint16_t>(terms_of(m, ta.n, ta.n));
+      dm[c] = static_cast<uint16_t>(m | TAIL);
+    }
+    __syncthreads();
+    while (true) {
+      topk_sort(val, dm, total);
+      kept = min(total, ta.k);
+      const double theta = kept == ta.k ? __longlong_as_double(val[kept - 1]) : 0.0;
+      if (tid == 0) {
+        n_act = 0;
+        cnt = kept;
+      }
+      __syncthreads();
+      for (int e = tid; e < kept; e += TOPK_THREADS)
+        if (dm[e] & TAIL) act[atomicAdd(&n_act, 1)] = static_cast<uint16_t>(e);
+      __syncthreads();
+      const int A = n_act;
+      if (A == 0) break;
+      const int pops = (cap - kept) / A;  // per diagonal, at most: their values fit
+      for (int c = tid; c < A; c += TOPK_THREADS) {
+        const int e0 = act[c], m = dm[e0] & 0x1fff;
+        dm[e0] = static_cast<uint16_t>(m);
+        double alpha = __longlong_as_double(val[e0]), sg[PN_MAX_P];
+#pragma unroll
+        for (int q = 0; q < PN_MAX_P; ++q)
+          sg[q] = q < ta.n_p ? sig[(int64_t)q * ta.nz + m] : 0.0;
+        int rem = left[m];
+        int at = -1;
+        for (int t = 0; t < pops; ++t) {
+          // sigma^(p)_m -= alpha^p for every p, and the largest stable p
+          --rem;
+          double pw = alpha, sv = 0.0;
+          int lg = 0, pl = -1;
+#pragma unroll
+          for (int q = 0; q < PN_MAX_P; ++q) {
+            if (q < ta.n_p) {
+              for (; lg < ta.p_log2[q]; ++lg) pw = __dmul_rn(pw, pw);
+              sg[q] = __dsub_rn(sg[q], pw);
+              if (sg[q] >= ta.tau) {
+                sv = sg[q];
+                pl = lg;
+              }
+            }
+          }
+          const double e = rem > 0 && pl >= 0 ? fmin(root_fp64(sv, pl), alpha) : 0.0;
+          if (!(e > 0.0) || e < theta) {  // the diagonal makes no more of the k values
+            at = -1;
+            break;
+          }
+          at = atomicAdd(&cnt, 1);
+          val[at] = __double_as_longlong(e);
+          dm[at] = static_cast<uint16_t>(m);
+          alpha = e;
+        }
+        if (at >= 0) {
+          dm[at] = static_cast<uint16_t>(m | TAIL);
+          left[m] = static_cast<uint16_t>(rem);
+#pragma unroll
+          for (int q = 0; q < PN_MAX_P; ++q)
+            if (q < ta.n_p) sig[(int64_t)q * ta.nz + m] = sg[q];
+        }
+      }
+      __syncthreads();
+      total = cnt;
+      __syncthreads();
+    }
+  }
+  for (int t = tid; t < ta.k; t += TOPK_THREADS) {
+    diag[t] = t < kept ? (dm[t] & 0x1fff) : -1;
+    if (dir == 0)
+      ta.vals[(int64_t)b * ta.ldk + t] =
+          t < kept ? static_cast<float>(__longlong_as_double(val[t]) * scale) : 0.0f;
   }
 }
 
@@ -1141,8 +1571,24 @@ int launch_topk(const TopkArgs& ta0, uint8_t* ws, void* stream) {
   const int smem_pop = nb * 8;
   if ((e = cudaFuncSetAttribute(k_topk_pop, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pop)))
     return e;
-  k_topk_sums<<<2 * ta.batch, FFT_THREADS, smem_sums, s>>>(ta);
-  k_topk_pop<<<2 * ta.batch, 32, smem_pop, s>>>(ta);
+  // threads: two groups of eight values each in the first pass; as many CTAs
+  // as fit on the SMs, each with a run of the work items
+  const int threads = N / 16 < 64 ? 64 : N / 16 > FFT_THREADS ? FFT_THREADS : N / 16;
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_topk_sums, threads, smem_sums)))
+    return e;
+  const int64_t items = (int64_t)2 * ta.batch * ta.n_p;
+  const int64_t room = static_cast<int64_t>(host_device_sms()) * (per_sm > 0 ? per_sm : 1);
+  k_topk_sums<<<static_cast<unsigned>(items < room ? items : room), threads, smem_sums, s>>>(ta);
+  if (ta.k <= TOPK_KMAX) {
+    const int smem = topk_merge_smem(ta.nz, ta.k);
+    if ((e = cudaFuncSetAttribute(k_topk_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
+      return e;
+    k_topk_merge<<<2 * ta.batch, TOPK_THREADS, smem, s>>>(ta);
+  } else {
+    k_topk_first<<<2 * ta.batch, FFT_THREADS, 0, s>>>(ta);
+    k_topk_pop<<<2 * ta.batch, 32, smem_pop, s>>>(ta);
+  }
   k_topk_index<<<ta.batch, 256, 0, s>>>(ta);
   return cudaGetLastError();
 }
