@@ -340,6 +340,34 @@ Level make_level(const Layout& L, const pn_opts* o, uint8_t* ws, const Schedule&
   return lv;
 }
 
+// Tile width of the one-launch product (k_fused_product), 0 for the level
+// launches.  It takes outputs of at most one tile per SM (128 x 64, or 128 x
+// 128) whose build time per level, 32 columns of K at a time, stays below
+// FUSED_NS: the level launches' images are built once per operand block over
+// all SMs, so they win on long contractions, but a call of theirs is 23
+// launches, about 100 us with their host time.  Nanoseconds per 32 columns,
+// maxima and one level, at 64 / 128 wide tiles (measured, K = 1024 .. 2048):
+// tensor copies (16-byte aligned rows): 3xTF32 1450 / 2010, 16-bit 1020 / 1080,
+// E4M3 1150 / 1460; unaligned rows: 2130 / 4050, 1700 / 2710, 1980 / 3420; TF32
+// as 3xTF32.  Level launches -> one launch: 256^3 3xTF32 (P = {1..128}) 94 -> 30
+// us, 512^3 117 -> 35, 1024^3 99 -> 58, 1024 x 2048 x 1536 BF16 92 -> 66, the
+// 512-vertex closure 1712 -> 1055.
+constexpr int64_t FUSED_NS = 55000;
+int fused_bn(const pn_opts* o, int64_t M, int64_t N, int64_t K, bool aligned, int sms) {
+  if (o->tile_m || o->tile_n || o->scaling == 1 || o->correction == 2 || o->estimator == 2 ||
+      o->debug_flags || host_tuned_bn(o->compute, M, N, K))
+    return 0;
+  const int64_t rows = ceil_div(M, TILE_M);
+  const int bn = rows * ceil_div(N, 64) <= sms ? 64 : rows * ceil_div(N, 128) <= sms ? 128 : 0;
+  if (bn == 0) return 0;
+  const int kind = o->compute == PN_F32_EXACT || o->compute == PN_TF32 ? 0
+                   : o->compute == PN_E4M3                             ? 2
+                                                                       : 1;
+  constexpr int ns[2][3][2] = {{{2130, 4050}, {1700, 2710}, {1980, 3420}},
+                               {{1450, 2010}, {1020, 1080}, {1150, 1460}}};
+  return ceil_div(K, 32) * ns[aligned ? 1 : 0][kind][bn == 128 ? 1 : 0] <= FUSED_NS ? bn : 0;
+}
+
 // The product proper, arguments already checked.
 pn_status run_pnorm(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
                     int64_t ldb, float* C, int64_t ldc, uint8_t* p_sel, float* S_sel,
@@ -351,6 +379,29 @@ pn_status run_pnorm(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda
   cm.post = post;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (K == 0) return cuda_status(launch_fill_empty(cm, o->p_log2[0], stream));
+  const bool aligned = (lda & 3) == 0 && (ldb & 3) == 0 &&
+                       ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+  if (const int bn = fused_bn(o, M, N, K, aligned, sms)) {
+    Prob& P = cm.single;
+    P.tiles_n = static_cast<int32_t>(ceil_div(N, bn));
+    P.state_ld = P.tiles_n * (bn / 32);  // at most the layout's
+    cm.BN = bn;
+    cm.cg = 1;
+    cm.total_tiles = P.tiles_m * P.tiles_n;
+    FusedArgs fa;
+    std::memset(&fa, 0, sizeof(fa));
+    fa.n_p = o->n_p;
+    for (int q = 0; q < o->n_p; ++q) fa.p_log2[q] = o->p_log2[q];
+    fa.estimator = o->estimator;
+    // APSP with the clamp: X_ii = 1 and X <= 1, so every maximum is 1
+    fa.unit_scales = post == 2 && o->scaling == 2;
+    if (o->ev_gemm_begin && cudaEventRecord(static_cast<cudaEvent_t>(o->ev_gemm_begin), s))
+      return PN_ECUDA;
+    if (launch_fused(cm, fa, stream)) return PN_ECUDA;
+    if (o->ev_gemm_end && cudaEventRecord(static_cast<cudaEvent_t>(o->ev_gemm_end), s))
+      return PN_ECUDA;
+    return PN_OK;
+  }
   int e = cudaMemsetAsync(ws, 0, L.ctrl_bytes, s);
   if (e) return PN_ECUDA;
   if ((e = launch_maxes(cm, stream))) return PN_ECUDA;

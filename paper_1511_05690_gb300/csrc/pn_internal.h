@@ -160,6 +160,15 @@ struct GroupedRun {
   int32_t* level_done;   // [n_slots]: CTAs that finished the slot
 };
 
+// A small product in one launch (k_fused_product): every level of P, largest
+// first, on one CTA per 128 x BN output tile.
+struct FusedArgs {
+  int32_t n_p;
+  int32_t p_log2[PN_MAX_P];
+  int32_t estimator;     // 0 or 1
+  int32_t unit_scales;   // every row and column maximum is known to be 1
+};
+
 // The level schedule: every p of P from the largest down, each followed --
 // for the r = 2 projection (estimator 2) -- by an extra "half" level at
 // 3p/4 when p/2 and p/4 are the two p below it in P.  Slot t runs level
@@ -292,6 +301,9 @@ struct NoMaps {};
 // if the driver's encoder is unavailable or the region is out of range.
 bool encode_img_rows(TensorMapBytes& out, const void* base, int64_t bytes, int box_rows = 128);
 void make_operand_maps(const Common& cm, OperandMaps& maps);
+// The maps of k_fused_product: boxes of 128 rows x raw_k columns of A (rows of
+// 128 bytes, swizzled) and of raw_k rows x cm.BN columns of B.
+void make_raw_maps(const Common& cm, int raw_k, OperandMaps& maps);
 
 int launch_maxes(const Common& cm, void* stream);
 // Grouped top level (scaling 0 or 2): maxima, domain test, scales and images
@@ -302,6 +314,7 @@ int launch_power_a(const Common& cm, const Level& lv, void* stream,
 int launch_power_b(const Common& cm, const Level& lv, void* stream,
                    const OperandMaps* maps = nullptr);
 int launch_gemm_level(const Common& cm, const Level& lv, int num_sms, void* stream);
+int launch_fused(const Common& cm, const FusedArgs& fa, void* stream);
 int launch_exact(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
                  int64_t ldb, float* C, int64_t ldc, int semiring, int variant, void* stream);
 int launch_fill_empty(const Common& cm, int plog0, void* stream);

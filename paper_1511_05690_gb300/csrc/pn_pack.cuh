@@ -87,7 +87,9 @@ struct Packer<MODE_3XTF32> {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      h[i] = tf32_bits(v[i]);
+      // the rounding of cvt.rna in two integer operations, which the ALU
+      // issues faster (a NaN may become a zero here, but then lo is a NaN)
+      h[i] = (__float_as_uint(v[i]) + 0x1000u) & 0xffffe000u;
       l[i] = tf32_bits(v[i] - __uint_as_float(h[i]));  // exact difference, then rounded
     }
     hi = make_uint4(h[0], h[1], h[2], h[3]);

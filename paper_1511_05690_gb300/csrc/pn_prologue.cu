@@ -343,15 +343,6 @@ __device__ __forceinline__ void lds_rotated(const float* src, int rot, float* v)
   }
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* map, int x, int y,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
-      "%3}], [%4];" ::"r"(dst_smem),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-
 template <int MODE, bool IS_B>
 __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B>::CTAS)
     k_image_tma(const __grid_constant__ Common cm, const __grid_constant__ Level lv,
@@ -665,9 +656,10 @@ EncodeTiledFn encode_tiled() {
 }
 
 // Row-major FP32 matrix of rows x cols with row pitch ld (elements) as a 2-D
-// tensor map with box box_rows x box_cols, zeros outside the matrix.
+// tensor map with box box_rows x box_cols, zeros outside the matrix; swizzle:
+// rows of 128 bytes with their 16-byte groups XORed by the row modulo 8.
 bool encode_fp32_2d(TensorMapBytes& out, const float* base, int64_t rows, int64_t cols, int64_t ld,
-                    int box_rows, int box_cols) {
+                    int box_rows, int box_cols, bool swizzle = false) {
   const EncodeTiledFn fn = encode_tiled();
   if (!fn || !base || rows < 1 || cols < 1 || ld < cols) return false;
   if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (ld & 3) != 0) return false;
@@ -679,7 +671,7 @@ bool encode_fp32_2d(TensorMapBytes& out, const float* base, int64_t rows, int64_
   const cuuint32_t estr[2] = {1, 1};
   return fn(reinterpret_cast<CUtensorMap*>(&out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
             const_cast<float*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -972,6 +964,12 @@ int launch_strips(const Common& cm, const Level& lv, void* stream) {
     case MODE_E4M3: return launch_strips_t<MODE_E4M3>(cm, lv, stream);
     default: return cudaErrorInvalidValue;
   }
+}
+
+void make_raw_maps(const Common& cm, int raw_k, OperandMaps& maps) {
+  const Prob& P = cm.single;
+  maps.has_a = encode_fp32_2d(maps.a, P.A, P.M, P.K, P.lda, TILE_M, raw_k, true) ? 1 : 0;
+  maps.has_b = encode_fp32_2d(maps.b, P.B, P.K, P.N, P.ldb, raw_k, cm.BN) ? 1 : 0;
 }
 
 int launch_maxes(const Common& cm, void* stream) {
