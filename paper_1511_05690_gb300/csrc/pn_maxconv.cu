@@ -3,18 +3,18 @@
 // Sec. 2.1).
 //
 // k_maxconv_fft: one CTA per problem, everything in shared memory.  Per p
-// (largest first): x' = x / max x and y' = y / max y raised to p in FP64, packed
-// as one complex sequence a = x'^p + i y'^p and transformed by one radix-2 FFT
-// (bit-reversed load, decimation in time); the spectra X, Y are separated from
-// A by Hermitian symmetry, Z = X Y, and the inverse FFT gives the ring
-// convolution S^(p) = x'^p * y'^p.  Each index m takes the first p with
-// S^(p)_m >= tau; z_m = max x max y (S^(p*)_m)^(1/p*).  The CTA stops as soon
-// as every index is resolved.  The transforms run in FP64: the FFT's absolute
-// error is about log2(N) 2^-53 times the norms of the powered vectors, which
-// is what the paper's tau = 1e-12 guards (GB300 issues FP64 at 1/64 of the
-// FP32 rate, so everything that needs no FP64 is kept out of it: the powers
-// x'^p are formed in FP32, relative error (p - 1) 2^-24, and the roots of
-// S >= 1e-30 by FP32 square roots).  When the indices still open after
+// (largest first): x' = x / max x and y' = y / max y raised to p in FP32
+// (relative error (p - 1) 2^-24), packed as one complex sequence
+// a = x'^p + i y'^p and transformed by one radix-2 FFT (decimation in time);
+// the spectra X, Y are separated from A by Hermitian symmetry, Z = X Y, and the
+// inverse FFT gives the ring convolution S^(p) = x'^p * y'^p.  Each index m takes
+// the first p with S^(p)_m >= tau; z_m = max x max y (S^(p*)_m)^(1/p*).  The CTA
+// stops as soon as every index is resolved.  An FFT's absolute error goes with
+// the norms of the powered vectors (about log2(N) 2^-53 of them in FP64), which
+// is what the paper's tau = 1e-12 guards.  GB300 issues FP64 at 1/64 of the
+// FP32 rate, so the transforms run in two floats per value, and the indices
+// whose sums are so small that their error would show get FP64 sums (below);
+// the roots of S >= 1e-30 are FP32 square roots.  When the indices still open after
 // a level hold few terms in total (typically the edges of the convolution),
 // their p-sums for every remaining p are summed directly in FP64 (the naive
 // ring convolution, which the FFT only reproduces) instead of running more
@@ -42,6 +42,7 @@ constexpr int FFT_NMAX = 1 << FFT_LOG_NMAX;
 // exp(-2 pi i k / NMAX), k < NMAX / 2; a transform of length N uses every
 // (NMAX / N)-th entry.
 __device__ double2 g_twiddle[FFT_NMAX / 2];
+__device__ float4 g_twiddle_ff[FFT_NMAX / 2];  // the same in two floats per part (cff)
 
 __global__ void k_twiddle_init() {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -49,15 +50,17 @@ __global__ void k_twiddle_init() {
   double s, c;
   sincospi(-2.0 * static_cast<double>(k) / FFT_NMAX, &s, &c);
   g_twiddle[k] = make_double2(c, s);
+  const float ch = static_cast<float>(c), sh = static_cast<float>(s);
+  g_twiddle_ff[k] = make_float4(ch, sh, static_cast<float>(c - ch), static_cast<float>(s - sh));
 }
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+  return make_double2(fma(a.x, b.x, -__dmul_rn(a.y, b.y)), fma(a.x, b.y, __dmul_rn(a.y, b.x)));
 }
 
 // conj(a) * b
 __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -a.y * b.x));
+  return make_double2(fma(a.x, b.x, __dmul_rn(a.y, b.y)), fma(a.x, b.y, -__dmul_rn(a.y, b.x)));
 }
 
 // In-place radix-2 decimation-in-time FFT of a[0..L) (L = 2^logL) held in
@@ -69,7 +72,7 @@ __device__ void fft_dit(double2* a, const double2* tw, int logL, int tws) {
   const int L = 1 << logL;
   int s0 = 0;
   if (logL >= 2) {
-    for (int g = threadIdx.x; g < (L >> 2); g += FFT_THREADS) {
+    for (int g = threadIdx.x; g < (L >> 2); g += static_cast<int>(blockDim.x)) {
       double2* q = a + 4 * g;
       const double2 a0 = q[0], a1 = q[1], a2 = q[2], a3 = q[3];
       const double2 b0 = make_double2(a0.x + a1.x, a0.y + a1.y);
@@ -89,7 +92,7 @@ __device__ void fft_dit(double2* a, const double2* tw, int logL, int tws) {
   for (int s = s0; s < logL; ++s) {
     const int h = 1 << s;                     // half span
     const int step = ((L >> 1) >> s) * tws;   // twiddle stride: L / (2h)
-    for (int b = threadIdx.x; b < (L >> 1); b += FFT_THREADS) {
+    for (int b = threadIdx.x; b < (L >> 1); b += static_cast<int>(blockDim.x)) {
       const int j = b & (h - 1);
       const int i0 = ((b >> s) << (s + 1)) + j;
       const int i1 = i0 + h;
@@ -173,7 +176,7 @@ __device__ void fft_dif(double2* a, const double2* tw, int logL, int tws) {
   for (int s = logL - 1; s >= 0; --s) {
     const int h = 1 << s;
     const int step = ((L >> 1) >> s) * tws;
-    for (int b = threadIdx.x; b < (L >> 1); b += FFT_THREADS) {
+    for (int b = threadIdx.x; b < (L >> 1); b += static_cast<int>(blockDim.x)) {
       const int j = b & (h - 1);
       const int i0 = ((b >> s) << (s + 1)) + j;
       const int i1 = i0 + h;
@@ -206,12 +209,13 @@ __device__ __forceinline__ int bitrev(int k, int logN) {
   return logN == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - logN));
 }
 
+__device__ __forceinline__ float pow_f32(float v, int plog) {
+  for (int s = 0; s < plog; ++s) v *= v;
+  return v;
+}
+
 // One level of the FFT convolution in shared memory: a = x'^p + i y'^p (zero
-// padded; powers in FP32, or in FP64 with POW64, which the NormQueue needs:
-// it subtracts the popped term's p-th power from the sums, so their error
-// must stay far below the next term's; y_rev reads y backwards), forward FFT
-// of length N,
-// the spectrum of the ring convolution, inverse at half length.  On return
+// padded; powers in FP32), forward FFT of length N, the spectrum of the ring convolution, inverse at half length.  On return
 // S_m = (m odd ? a[m/2].y : a[m/2].x) * 2 / N.
 //
 // The spectrum: X_k = (A_k + conj A_(N-k)) / 2, Y_k = (A_k - conj A_(N-k)) /
@@ -222,22 +226,14 @@ __device__ __forceinline__ int bitrev(int k, int logN) {
 // V_k = E_k + i O_k = (Z_k + conj Z_(M-k)) / 2 + i W^-k (Z_k - conj Z_(M-k)) / 2
 // is the DFT of v_j = S_2j + i S_(2j+1).  Thread work: k and M - k together
 // (reads A at k, N - k, M - k, M + k).
-template <bool POW64>
 __device__ void conv_level(double2* a, const double2* tw, const MaxconvArgs& ma, const float* x,
-                           const float* y, double isx, double isy, int plog, bool y_rev) {
+                           const float* y, float isx, float isy, int plog) {
   const int N = 1 << ma.logN;
-  const int tid = threadIdx.x;
-  using T = typename std::conditional<POW64, double, float>::type;
-  for (int k = tid; k < N; k += FFT_THREADS) {
-    T xr = 0, yr = 0;
-    if (k < ma.nx) {
-      xr = static_cast<T>(x[k]) * static_cast<T>(isx);
-      for (int s = 0; s < plog; ++s) xr *= xr;
-    }
-    if (k < ma.ny) {
-      yr = static_cast<T>(y[y_rev ? ma.ny - 1 - k : k]) * static_cast<T>(isy);
-      for (int s = 0; s < plog; ++s) yr *= yr;
-    }
+  const int tid = threadIdx.x, nt = static_cast<int>(blockDim.x);
+  for (int k = tid; k < N; k += nt) {
+    float xr = 0.0f, yr = 0.0f;
+    if (k < ma.nx) xr = pow_f32(x[k] * isx, plog);
+    if (k < ma.ny) yr = pow_f32(y[k] * isy, plog);
     a[bitrev(k, ma.logN)] = make_double2(static_cast<double>(xr), static_cast<double>(yr));
   }
   __syncthreads();
@@ -246,7 +242,7 @@ __device__ void conv_level(double2* a, const double2* tw, const MaxconvArgs& ma,
   constexpr int QUADS = FFT_NMAX / 4 / FFT_THREADS + 1;
   double2 vk[QUADS], vm[QUADS];
   for (int u = 0; u < QUADS; ++u) {
-    const int k = tid + u * FFT_THREADS;
+    const int k = tid + u * nt;
     if (k <= (M >> 1)) {
       const double2 zk = spec_z(a[k], a[(N - k) & (N - 1)]);
       const double2 zm = spec_z(a[M - k], a[M + k]);
@@ -256,7 +252,7 @@ __device__ void conv_level(double2* a, const double2* tw, const MaxconvArgs& ma,
   }
   __syncthreads();
   for (int u = 0; u < QUADS; ++u) {
-    const int k = tid + u * FFT_THREADS;
+    const int k = tid + u * nt;
     if (k <= (M >> 1)) {
       a[bitrev(k, ma.logN - 1)] = vk[u];
       if (k != 0 && (M - k) != k) a[bitrev(M - k, ma.logN - 1)] = vm[u];
@@ -266,29 +262,417 @@ __device__ void conv_level(double2* a, const double2* tw, const MaxconvArgs& ma,
   fft_dit<true>(a, tw, ma.logN - 1, 2);
 }
 
-__global__ void __launch_bounds__(FFT_THREADS, 1)
+// ---- transforms in registers.  The same radix-2 butterflies, twiddles and
+// operation order as fft_dit / conv_level (in FP64 every value has the same
+// bits), but eight values per thread stay in registers for three stages, so a
+// transform of 2^13 makes 9 passes over shared memory with a barrier each
+// instead of 28, and nothing is permuted: the forward transform reads natural
+// order and leaves frequency k at address bitrev(k); the last forward stage
+// pairs the addresses of k and k + N/2, which the spectrum needs together
+// with those of N - k and N/2 - k, so it is fused into the spectrum; the
+// spectrum's half-length sequence, left in the even addresses in
+// bit-reversed order, is what the decimation in time starts from.
+//
+// Values are double2, or cff, each part the unevaluated sum of two floats: an
+// addition (8 FP32 operations) and a product (4) keep about 2^-46 of their
+// operands' magnitude, and GB300 issues 64 FP32 operations per FP64 one, so a
+// butterfly takes 64 lane slots instead of 8 x 64.
+// What bounds the double2 form is the FP64 issue rate (two lanes per clock and
+// SM): about 6.8e5 FP64 instructions per level at N = 2^13.
+
+// Shared-memory slot of element i: bits 1-2 are XORed with bits 4-5, so that
+// the passes with a stride of two or eight elements spread over the banks.
+__device__ __forceinline__ int slot(int i) { return i ^ (((i >> 4) & 3) << 1); }
+
+// A complex value in two floats per part: h = (x.h, y.h), l = (x.l, y.l), each
+// pair one operand of the packed FP32 instructions (two operations, rounded
+// as by themselves, in one issue slot; the kernel runs out of slots and of
+// instruction cache, not of FP32 lanes).
+struct alignas(16) cff {
+  uint64_t h, l;
+};
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+constexpr uint64_t F2_NEG = 0xbf800000bf800000ull;  // (-1, -1)
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) { return f2_fma(b, F2_NEG, a); }
+__device__ __forceinline__ uint64_t f2_neg(uint64_t a) { return a ^ 0x8000000080000000ull; }
+
+// a + b: the rounding error of the high parts by Knuth's two-sum, the low parts
+// added to it (not renormalised).
+__device__ __forceinline__ cff ff_add(uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl) {
+  const uint64_t s = f2_add(ah, bh), t = f2_sub(s, ah);
+  const uint64_t e = f2_add(f2_sub(ah, f2_sub(s, t)), f2_sub(bh, t));
+  return cff{s, f2_add(e, f2_add(al, bl))};
+}
+// a - b
+__device__ __forceinline__ cff ff_sub(uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl) {
+  const uint64_t s = f2_sub(ah, bh), t = f2_sub(s, ah);
+  const uint64_t e = f2_sub(f2_sub(ah, f2_sub(s, t)), f2_add(bh, t));
+  return cff{s, f2_add(e, f2_sub(al, bl))};
+}
+
+__device__ __forceinline__ double2 c_add(double2 a, double2 b) {
+  return make_double2(a.x + b.x, a.y + b.y);
+}
+__device__ __forceinline__ double2 c_sub(double2 a, double2 b) {
+  return make_double2(a.x - b.x, a.y - b.y);
+}
+// a + conj b, a - conj b, a + i b, -i a
+__device__ __forceinline__ double2 c_add_conj(double2 a, double2 b) {
+  return make_double2(a.x + b.x, a.y - b.y);
+}
+__device__ __forceinline__ double2 c_sub_conj(double2 a, double2 b) {
+  return make_double2(a.x - b.x, a.y + b.y);
+}
+__device__ __forceinline__ double2 c_add_i(double2 a, double2 b) {
+  return make_double2(a.x - b.y, a.y + b.x);
+}
+__device__ __forceinline__ double2 c_mul_mi(double2 a) { return make_double2(a.y, -a.x); }
+__device__ __forceinline__ cff c_add(cff a, cff b) { return ff_add(a.h, a.l, b.h, b.l); }
+__device__ __forceinline__ cff c_sub(cff a, cff b) { return ff_sub(a.h, a.l, b.h, b.l); }
+__device__ __forceinline__ cff c_conj(cff a) {
+  return cff{a.h ^ 0x8000000000000000ull, a.l ^ 0x8000000000000000ull};
+}
+// i a = (-y, x)
+__device__ __forceinline__ cff c_muli(cff a) {
+  const float2 h = f2_unpack(a.h), l = f2_unpack(a.l);
+  return cff{f2_pack(-h.y, h.x), f2_pack(-l.y, l.x)};
+}
+__device__ __forceinline__ cff c_add_conj(cff a, cff b) { return c_add(a, c_conj(b)); }
+__device__ __forceinline__ cff c_sub_conj(cff a, cff b) { return c_sub(a, c_conj(b)); }
+__device__ __forceinline__ cff c_add_i(cff a, cff b) { return c_add(a, c_muli(b)); }
+__device__ __forceinline__ cff c_mul_mi(cff a) {
+  const cff b = c_muli(a);
+  return cff{f2_neg(b.h), f2_neg(b.l)};
+}
+// w v = v.x (w.x, w.y) + v.y (-w.y, w.x)
+__device__ __forceinline__ cff cmul(cff w, cff v) {
+  const cff iw = c_muli(w);
+  const float2 vh = f2_unpack(v.h), vl = f2_unpack(v.l);
+  const uint64_t xh = f2_pack(vh.x, vh.x), xl = f2_pack(vl.x, vl.x);
+  const uint64_t yh = f2_pack(vh.y, vh.y), yl = f2_pack(vl.y, vl.y);
+  const uint64_t p = f2_mul(xh, w.h), q = f2_mul(yh, iw.h);
+  uint64_t e = f2_fma(xh, w.h, f2_neg(p)), f = f2_fma(yh, iw.h, f2_neg(q));
+  e = f2_fma(xh, w.l, f2_fma(xl, w.h, e));
+  f = f2_fma(yh, iw.l, f2_fma(yl, iw.h, f));
+  return ff_add(p, e, q, f);
+}
+__device__ __forceinline__ cff cmulc(cff w, cff v) { return cmul(c_conj(w), v); }
+
+// Twiddle k of the table.  The two-float table is stored with the low three
+// index bits XORed with the higher ones, three at a time: the passes read it
+// with strides of powers of two, which would meet in a few banks (the FP64
+// form has time for that: its arithmetic takes eight times as long).
+__device__ __forceinline__ int tw_slot(int k) {
+  return k ^ (((k >> 3) ^ (k >> 6) ^ (k >> 9)) & 7);
+}
+__device__ __forceinline__ double2 tw_at(const double2* tw, int k) { return tw[k]; }
+__device__ __forceinline__ cff tw_at(const cff* tw, int k) { return tw[tw_slot(k)]; }
+
+template <typename C>
+__device__ __forceinline__ void bfly(C& u, C& v, C t) {
+  const C a = u;
+  u = c_add(a, t);
+  v = c_sub(a, t);
+}
+
+// The butterfly with the twiddle -i.  (A negated FP64 value costs an FP64
+// instruction unless it is the subtrahend of the operation that uses it.)
+__device__ __forceinline__ void bfly_mi(double2& u, double2& v) {
+  const double2 a = u, b = v;
+  u = make_double2(a.x + b.y, a.y - b.x);
+  v = make_double2(a.x - b.y, a.y + b.x);
+}
+
+// R stages s .. s + R - 1 of a transform of 2^lg values on the 2^R values
+// v[r] of one group; v[r] sits at position j + (r << s) within its block of
+// 2^(s + R) (positions as in fft_dit).  tw[k << tsh] = exp(-2 pi i k / 2^lg).
+template <int R, bool INV, typename C>
+__device__ __forceinline__ void group_stages(C (&v)[1 << R], const C* tw, int lg, int tsh, int s,
+                                             int j) {
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+    const int sh = lg - 1 - s - t + tsh;
+#pragma unroll
+    for (int o = 0; o < (1 << t); ++o) {
+      const C w = tw_at(tw, (j + (o << s)) << sh);
+#pragma unroll
+      for (int r = 0; r < (1 << R); r += 2 << t) {
+        const C b = v[r + o + (1 << t)];
+        bfly(v[r + o], v[r + o + (1 << t)], INV ? cmulc(w, b) : cmul(w, b));
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ int rev_bits(int k, int n) {
+  return n == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - n));
+}
+
+// Forward stages s .. s + R - 1 in place: the address of a position is its bit
+// reversal, so stage t pairs addresses that differ in bit lg - 1 - t.
+template <int R, typename C>
+__device__ __forceinline__ void fwd_pass(C* a, const C* tw, int lg, int s) {
+  const int low = lg - s - R;  // address bits below the group's
+  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+    const int hi = g >> low, base = (hi << (low + R)) | (g & ((1 << low) - 1));
+    C v[1 << R];
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(base + (rev_bits(r, R) << low))];
+    group_stages<R, false>(v, tw, lg, 0, s, rev_bits(hi, s));
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) a[slot(base + (rev_bits(r, R) << low))] = v[r];
+  }
+  __syncthreads();
+}
+
+// Inverse stages s .. s + R - 1 of the 2^lg values in the even addresses.
+template <int R, typename C>
+__device__ __forceinline__ void inv_pass(C* a, const C* tw, int lg, int s) {
+  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+    const int j = g & ((1 << s) - 1), base = ((g >> s) << (s + R)) | j;
+    C v[1 << R];
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(2 * (base + (r << s)))];
+    group_stages<R, true>(v, tw, lg, 1, s, j);
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) a[slot(2 * (base + (r << s)))] = v[r];
+  }
+  __syncthreads();
+}
+
+// The spectrum from the packed pair's transform (all but its last stage done)
+// to the half-length sequence 8 V_k in the even addresses; see conv_level.
+// The halves of the formulas there are left out: a power of two, exact.
+template <typename C>
+__device__ __forceinline__ void spectrum_pass(C* a, const C* tw, int lg) {
+  const int lm = lg - 1, M = 1 << lm;
+  for (int e = threadIdx.x; e <= (M >> 1); e += blockDim.x) {
+    // p = bitrev(k): 0, then the lower half of every [2^h, 2^(h + 1)); the
+    // address of M - k mirrors p within that range
+    int p = e, pm = e;
+    if (e > 1) {
+      const int f = e - 1, hb = 1 << (31 - __clz(f));
+      p = f + hb;
+      pm = p ^ (2 * hb - 1);
+    }
+    const int k = rev_bits(p, lm);
+    C ak = a[slot(2 * p)], amk = a[slot(2 * p + 1)];  // frequencies k, k + M
+    const C wk = tw_at(tw, k);
+    bfly(ak, amk, cmul(wk, amk));
+    C am = ak, an = amk;                              // M - k, N - k
+    if (k == 0) {
+      an = ak;  // N - 0 = 0 and M - 0 = M
+      am = amk;
+    } else if (pm != p) {
+      am = a[slot(2 * pm)];
+      an = a[slot(2 * pm + 1)];
+      bfly(am, an, cmul(tw_at(tw, M - k), an));
+    }
+    auto z4 = [](C u, C v) {  // 4 spec_z: (u + conj v) (-i (u - conj v))
+      return cmul(c_add_conj(u, v), c_mul_mi(c_sub_conj(u, v)));
+    };
+    auto v8 = [](C zk, C zm, C w) {  // 8 spec_v
+      return c_add_i(c_add_conj(zk, zm), cmulc(w, c_sub_conj(zk, zm)));
+    };
+    const C zk = z4(ak, an), zm = z4(am, amk);
+    a[slot(2 * p)] = v8(zk, zm, wk);
+    if (k != 0 && pm != p) a[slot(2 * pm)] = v8(zm, zk, tw_at(tw, M - k));
+  }
+  __syncthreads();
+}
+
+// The passes after the first forward stages (s of them done): the rest of the
+// forward transform, the spectrum, the inverse.  On return S_m = 8 N / 2 times
+// part m & 1 of a[slot(m & ~1)].  Three stages per pass in FP64; two in two
+// floats, whose butterflies are five times as many instructions: with three, a
+// pass's loop outgrows the instruction cache (a third of the fetches missed)
+// and its registers allow half the warps.
+__device__ __forceinline__ void conv_passes(double2* a, const double2* tw, int lg, int s) {
+  for (; s + 3 <= lg - 1; s += 3) fwd_pass<3>(a, tw, lg, s);
+  if (s + 2 == lg - 1) fwd_pass<2>(a, tw, lg, s);
+  else if (s + 1 == lg - 1) fwd_pass<1>(a, tw, lg, s);
+  spectrum_pass(a, tw, lg);
+  const int lm = lg - 1;
+  for (s = 0; s + 3 <= lm; s += 3) inv_pass<3>(a, tw, lm, s);
+  if (s + 2 == lm) inv_pass<2>(a, tw, lm, s);
+  else if (s + 1 == lm) inv_pass<1>(a, tw, lm, s);
+}
+__device__ __forceinline__ void conv_passes(cff* a, const cff* tw, int lg) {
+  int s = (lg - 1) & 1;
+  if (s) fwd_pass<1>(a, tw, lg, 0);
+  for (; s < lg - 1; s += 2) fwd_pass<2>(a, tw, lg, s);
+  spectrum_pass(a, tw, lg);
+  const int lm = lg - 1;
+  s = lm & 1;
+  if (s) inv_pass<1>(a, tw, lm, 0);
+  for (; s < lm; s += 2) inv_pass<2>(a, tw, lm, s);
+}
+
+// Whether the remaining p-sums of open indices with W terms in all are cheaper
+// summed directly (about W (8 + 2 q) FP64 operations) than by one more FFT
+// level (about 10 N log2 N).
+__device__ __forceinline__ bool few_terms(unsigned long long W, int q, int logN) {
+  return W * static_cast<unsigned long long>(8 + 2 * q) <=
+         10ull * (1ull << logN) * static_cast<unsigned long long>(logN);
+}
+
+// Sum over a warp, the same on every lane.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// direct_levels by a whole warp: lanes take the terms in turn (an index at the
+// edge has a few dozen at most, and one FP64 instruction of a warp takes 64
+// cycles however many lanes it has).
+__device__ void direct_levels_warp(const MaxconvArgs& ma, const float* x, const float* y,
+                                   double isx, double isy, double sxy, int m, int q, float* z,
+                                   uint8_t* res, int lane) {
+  const int lo = m - ma.ny + 1 > 0 ? m - ma.ny + 1 : 0;
+  const int hi = m < ma.nx - 1 ? m : ma.nx - 1;
+  // level by level from the largest p left: most indices stop at the first
+  for (int u = q - 1; u >= 0; --u) {
+    double S = 0.0;
+    for (int i = lo + lane; i <= hi; i += 32) {
+      double t = (static_cast<double>(x[i]) * isx) * (static_cast<double>(y[m - i]) * isy);
+      for (int s = 0; s < ma.p_log2[u]; ++s) t *= t;
+      S += t;
+    }
+    S = warp_sum(S);
+    const bool stable = S >= ma.tau;
+    if (stable || u == 0) {
+      if (lane == 0) {
+        z[m] = static_cast<float>(sxy * root_pow2(S, ma.p_log2[u]));
+        res[m] = static_cast<uint8_t>(ma.p_log2[u] | (stable ? 0 : 0x80));
+      }
+      return;
+    }
+  }
+}
+
+// The levels q .. 0 of one problem by FP64 transforms, for the indices still
+// open in res (0xFF); block-wide.
+__device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw, uint8_t* res,
+                                 const float* x, const float* y, float isx, float isy, double sxy,
+                                 float* z, int q) {
+  __shared__ unsigned long long open_terms;
+  __shared__ int n_open;
+  const int N = 1 << ma.logN, tid = threadIdx.x, nt = static_cast<int>(blockDim.x);
+  const double invM = 2.0 / N;
+  __syncthreads();
+  for (int k = tid; k < (N >> 1); k += nt) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - ma.logN)];
+  for (; q >= 0; --q) {
+    const int plog = ma.p_log2[q];
+    conv_level(a, tw, ma, x, y, isx, isy, plog);
+    // selection: first (largest) p with S >= tau; the smallest p takes the rest
+    if (tid == 0) {
+      open_terms = 0ull;
+      n_open = 0;
+    }
+    __syncthreads();
+    unsigned long long my_terms = 0ull;
+    for (int m = tid; m < ma.nz; m += nt) {
+      if (res[m] != 0xFF) continue;
+      const double S = ((m & 1) ? a[m >> 1].y : a[m >> 1].x) * invM;
+      const bool stable = S >= ma.tau;
+      if (stable || q == 0) {
+        z[m] = static_cast<float>(sxy * root_pow2(S, plog));
+        res[m] = static_cast<uint8_t>(plog | (stable ? 0 : 0x80));
+      } else {
+        my_terms += static_cast<unsigned long long>(terms_of(m, ma.nx, ma.ny));
+      }
+    }
+    if (my_terms) atomicAdd(&open_terms, my_terms);
+    __syncthreads();
+    const unsigned long long W = open_terms;
+    if (W == 0ull) break;
+    if (few_terms(W, q, ma.logN)) {
+      // compact list of the open indices (the FFT buffer is free now)
+      int* list = reinterpret_cast<int*>(a);
+      for (int m = tid; m < ma.nz; m += nt)
+        if (res[m] == 0xFF) list[atomicAdd(&n_open, 1)] = m;
+      __syncthreads();
+      const int cnt = n_open;
+      for (int e = tid; e < cnt; e += nt)
+        direct_levels(ma, x, y, static_cast<double>(isx), static_cast<double>(isy), sxy, list[e],
+                      q, z, res);
+      break;
+    }
+  }
+}
+
+// One CTA per problem.  Per level the transforms run in two floats per value
+// (see above).  Their rounding adds noise to every S_m, independent of S_m's
+// own size: with R the root mean square of the S_m, its standard deviation is
+// at most sigma = 2^-45 sqrt(log2 N) R (measured 0.12 to 0.28 sigma, largest
+// value 1.2 sigma, N = 2^13), that of FP64 transforms sigma64 = 2^-53
+// sqrt(log2 N) R (measured 0.6).  An index with S_m >= theta = 2^28 sigma (16
+// sigma below 2^-24 of S_m) is rooted from it.  The others -- the outermost few,
+// which sum few terms -- get S_m by a direct FP64 sum, which has no such noise.
+// Where that sum lies within 3 sigma64 of tau (about one problem in 400), or
+// where too many indices lie below theta (wide ranges of values), the
+// problem's level and the rest run in FP64 transforms, so that p_sel is what
+// FP64 transforms give.
+// Per problem of n = 4096 (one CTA, P = {1..64}): 62 us, of which the transforms
+// take 37 (issue slots: about 50 instructions per butterfly), against 240 by
+// FP64 transforms at 78 % of the FP64 pipe; 1024 problems 0.60 ms (0.43 where no
+// problem falls back to FP64), by FP64 transforms 1.66.
+constexpr int MC_THREADS = 1024;
+constexpr int FF_SMALL_MAX = 512;  // indices summed directly, at most
+__global__ void __launch_bounds__(MC_THREADS, 1)
     k_maxconv_fft(const __grid_constant__ MaxconvArgs ma) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N = 1 << ma.logN;
-  double2* a = reinterpret_cast<double2*>(smem);
-  double2* tw = a + N;
+  const int lg = ma.logN, N = 1 << lg;
+  cff* a = reinterpret_cast<cff*>(smem);
+  cff* tw = a + N;
   uint8_t* res = reinterpret_cast<uint8_t*>(tw + (N >> 1));  // p_sel, 0xFF = open
-  __shared__ double red[2][FFT_THREADS / 32];
+  __shared__ float red[2][MC_THREADS / 32];
+  __shared__ unsigned long long s_terms;
+  __shared__ int n_small, n_open, redo;
+  __shared__ int small[FF_SMALL_MAX];
+  __shared__ double small_S[FF_SMALL_MAX];
   const int b = blockIdx.x;
   const float* x = ma.x + (int64_t)b * ma.ldx;
   const float* y = ma.y + (int64_t)b * ma.ldy;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = static_cast<int>(blockDim.x), nw = nt >> 5;
 
-  for (int k = tid; k < (N >> 1); k += FFT_THREADS) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - ma.logN)];
+  for (int k = tid; k < (N >> 1); k += nt) 
+    *reinterpret_cast<float4*>(tw + tw_slot(k)) = g_twiddle_ff[k << (FFT_LOG_NMAX - lg)];
   // maxima and domain (R+, finite)
   float mx = 0.0f, my = 0.0f;
   bool bad = false;
-  for (int k = tid; k < ma.nx; k += FFT_THREADS) {
+  for (int k = tid; k < ma.nx; k += nt) {
     const float v = x[k];
     bad |= !(v >= 0.0f && v <= 3.4028235e38f);
     mx = fmaxf(mx, v);
   }
-  for (int k = tid; k < ma.ny; k += FFT_THREADS) {
+  for (int k = tid; k < ma.ny; k += nt) {
     const float v = y[k];
     bad |= !(v >= 0.0f && v <= 3.4028235e38f);
     my = fmaxf(my, v);
@@ -306,67 +690,157 @@ __global__ void __launch_bounds__(FFT_THREADS, 1)
     red[0][warp] = mx;
     red[1][warp] = my;
   }
-  for (int m = tid; m < ma.nz; m += FFT_THREADS) res[m] = 0xFF;
+  for (int m = tid; m < ma.nz; m += nt) res[m] = 0xFF;
   __syncthreads();
-  double sx = 0.0, sy = 0.0;
-  for (int w = 0; w < FFT_THREADS / 32; ++w) {
-    sx = fmax(sx, red[0][w]);
-    sy = fmax(sy, red[1][w]);
+  mx = my = 0.0f;
+  for (int w = 0; w < nw; ++w) {
+    mx = fmaxf(mx, red[0][w]);
+    my = fmaxf(my, red[1][w]);
   }
-  if (sx == 0.0) sx = 1.0;  // a zero vector keeps scale 1
-  if (sy == 0.0) sy = 1.0;
-  const double invM = 2.0 / N;
-  const float isx_f = static_cast<float>(1.0 / sx), isy_f = static_cast<float>(1.0 / sy);
-  const double sxy = sx * sy;
+  // the FP64 scalars by one warp (one FP64 instruction takes a warp 64 cycles)
+  __shared__ double s_sxy;
+  __shared__ float s_f[4];
+  if (warp == 0) {
+    // a zero vector keeps scale 1
+    const double sx = mx == 0.0f ? 1.0 : static_cast<double>(mx);
+    const double sy = my == 0.0f ? 1.0 : static_cast<double>(my);
+    const double p = sx * sy;
+    const float ph = static_cast<float>(p);
+    if (lane == 0) {
+      s_sxy = p;
+      s_f[0] = static_cast<float>(1.0 / sx);
+      s_f[1] = static_cast<float>(1.0 / sy);
+      s_f[2] = ph;
+      s_f[3] = static_cast<float>(p - ph);
+    }
+  }
+  __syncthreads();
+  const double sxy = s_sxy;
+  const float isx = s_f[0], isy = s_f[1], sxy_h = s_f[2], sxy_l = s_f[3];
   float* z = ma.z + (int64_t)b * ma.ldz;
-  __shared__ unsigned long long open_terms;
-  __shared__ int n_open;
-
-  for (int q = ma.n_p - 1; q >= 0; --q) {
+  const float scale = 0.25f / N;  // 2 / N, and the spectrum's 8
+  const float tau = static_cast<float>(ma.tau);
+  // products of the scales outside FP32's comfortable range, tiny transforms and
+  // thresholds beyond FP32: FP64 from the start
+  bool ff = lg >= 5 && sxy_h >= 1e-30f && sxy_h <= 1e30f && tau >= 1e-30f && tau <= 1e6f;
+  int q = ma.n_p - 1;
+  for (; ff && q >= 0; --q) {
     const int plog = ma.p_log2[q];
-    conv_level<false>(a, tw, ma, x, y, isx_f, isy_f, plog, false);
-    // selection: first (largest) p with S >= tau; the smallest p takes the rest
-    if (tid == 0) {
-      open_terms = 0ull;
-      n_open = 0;
+    for (int k = tid; k < N; k += nt) {
+      const float xr = k < ma.nx ? pow_f32(x[k] * isx, plog) : 0.0f;
+      const float yr = k < ma.ny ? pow_f32(y[k] * isy, plog) : 0.0f;
+      a[slot(k)] = cff{f2_pack(xr, yr), 0ull};
     }
     __syncthreads();
-    unsigned long long my_terms = 0ull;
-    for (int m = tid; m < ma.nz; m += FFT_THREADS) {
-      if (res[m] != 0xFF) continue;
-      const double S = ((m & 1) ? a[m >> 1].y : a[m >> 1].x) * invM;
-      const bool stable = S >= ma.tau;
-      if (stable || q == 0) {
-        z[m] = static_cast<float>(sxy * root_pow2(S, plog));
-        res[m] = static_cast<uint8_t>(plog | (stable ? 0 : 0x80));
-      } else {
-        my_terms += static_cast<unsigned long long>(terms_of(m, ma.nx, ma.ny));
+    conv_passes(a, tw, lg);
+    // the sums' root mean square
+    constexpr int PER = FFT_NMAX / MC_THREADS;
+    float S[PER], ss = 0.0f;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int m = tid + u * nt;
+      S[u] = 0.0f;
+      if (m < ma.nz) {
+        const cff v = a[slot(m & ~1)];
+        const float2 h = f2_unpack(v.h), l = f2_unpack(v.l);
+        S[u] = ((m & 1) ? __fadd_rn(h.y, l.y) : __fadd_rn(h.x, l.x)) * scale;
+        ss = fmaf(S[u], S[u], ss);
       }
     }
-    if (my_terms) atomicAdd(&open_terms, my_terms);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+    if (lane == 0) red[0][warp] = ss;
+    if (tid == 0) {
+      s_terms = 0ull;
+      n_small = n_open = redo = 0;
+    }
     __syncthreads();
-    const unsigned long long W = open_terms;
-    if (W == 0ull) break;
-    // few open terms: sum the remaining p directly (cost ~ W (8 + 2q) FP64
-    // operations against ~10 N log2 N for one more FFT level)
-    if (W * static_cast<unsigned long long>(8 + 2 * q) <=
-        10ull * static_cast<unsigned long long>(N) * static_cast<unsigned long long>(ma.logN)) {
-      // compact list of the open indices (the FFT buffer is free now)
-      int* list = reinterpret_cast<int*>(a);
-      for (int m = tid; m < ma.nz; m += FFT_THREADS)
-        if (res[m] == 0xFF) list[atomicAdd(&n_open, 1)] = m;
-      __syncthreads();
-      const int cnt = n_open;
-      for (int e = tid; e < cnt; e += FFT_THREADS)
-        direct_levels(ma, x, y, static_cast<double>(isx_f), static_cast<double>(isy_f), sxy,
-                      list[e], q, z, res);
+    ss = 0.0f;
+    for (int w = 0; w < nw; ++w) ss += red[0][w];
+    const float noise = sqrtf(static_cast<float>(lg) * ss / N);
+    const float theta = fmaxf(noise * 7.62939453e-6f, 4.0f * tau);           // 2^28 2^-45
+    const float near = noise * 3.33066907e-16f;  // 3 2^-53
+    unsigned long long terms = 0ull;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int m = tid + u * nt;
+      if (m >= ma.nz || res[m] != 0xFF) continue;
+      if (S[u] >= theta) {
+        float r = S[u];
+        for (int s = 0; s < plog; ++s) r = sqrtf(r);
+        z[m] = fmaf(sxy_h, r, sxy_l * r);
+        res[m] = static_cast<uint8_t>(plog);
+      } else {
+        const int at = atomicAdd(&n_small, 1);
+        if (at < FF_SMALL_MAX) small[at] = m;
+        terms += static_cast<unsigned long long>(terms_of(m, ma.nx, ma.ny));
+      }
+    }
+    if (terms) atomicAdd(&s_terms, terms);
+    __syncthreads();
+    const int cnt = n_small;
+    // too many terms to sum directly (against an FP64 level)
+    if (cnt > FF_SMALL_MAX || s_terms > 2ull * N) {
+      ff = false;
       break;
     }
+    __syncthreads();
+    if (tid == 0) s_terms = 0ull;
+    __syncthreads();
+    for (int e = warp; e < cnt; e += nw) {  // a warp per index
+      const int m = small[e];
+      const int lo = m - ma.ny + 1 > 0 ? m - ma.ny + 1 : 0, hi = m < ma.nx - 1 ? m : ma.nx - 1;
+      double t = 0.0;
+      for (int i = lo + lane; i <= hi; i += 32)
+        t = fma(static_cast<double>(pow_f32(x[i] * isx, plog)),
+                static_cast<double>(pow_f32(y[m - i] * isy, plog)), t);
+      t = warp_sum(t);
+      if (lane == 0) {
+        small_S[e] = t;
+        if (fabsf(static_cast<float>(t - ma.tau)) <= near) redo = 1;
+      }
+    }
+    __syncthreads();
+    if (redo) {
+      ff = false;
+      break;
+    }
+    terms = 0ull;
+    for (int e = tid; e < cnt; e += nt) {
+      const int m = small[e];
+      const double t = small_S[e];
+      const bool stable = t >= ma.tau;
+      if (stable || q == 0) {
+        z[m] = static_cast<float>(sxy * root_pow2(t, plog));
+        res[m] = static_cast<uint8_t>(plog | (stable ? 0 : 0x80));
+      } else {
+        terms += static_cast<unsigned long long>(terms_of(m, ma.nx, ma.ny));
+      }
+    }
+    if (terms) atomicAdd(&s_terms, terms);
+    __syncthreads();
+    const unsigned long long W = s_terms;
+    if (W == 0ull) break;
+    if (few_terms(W, q, lg)) {
+      int* list = reinterpret_cast<int*>(a);  // the FFT buffer is free now
+      for (int m = tid; m < ma.nz; m += nt)
+        if (res[m] == 0xFF) list[atomicAdd(&n_open, 1)] = m;
+      __syncthreads();
+      const int open = n_open;
+      for (int e = warp; e < open; e += nw)
+        direct_levels_warp(ma, x, y, static_cast<double>(isx), static_cast<double>(isy), sxy,
+                           list[e], q, z, res, lane);
+      break;
+    }
+    __syncthreads();
   }
+  if (!ff && q >= 0)
+    maxconv_levels64(ma, reinterpret_cast<double2*>(a), reinterpret_cast<double2*>(tw), res, x, y,
+                     isx, isy, sxy, z, q);
   __syncthreads();
   if (ma.psel) {
     uint8_t* ps = ma.psel + (int64_t)b * ma.ldp;
-    for (int m = tid; m < ma.nz; m += FFT_THREADS) ps[m] = res[m];
+    for (int m = tid; m < ma.nz; m += nt) ps[m] = res[m];
   }
 }
 
@@ -765,86 +1239,6 @@ __device__ __forceinline__ double pow_pow2(double a, int plog) {
   return a;
 }
 
-// ---- transforms of the p-sums.  The same radix-2 butterflies, twiddles and
-// operation order as fft_dit / conv_level (every p-sum has the same bits),
-// but eight values per thread stay in registers for three stages, so a
-// transform of 2^13 makes 9 passes over shared memory with a barrier each
-// instead of 28, and nothing is permuted: the forward transform reads natural
-// order and leaves frequency k at address bitrev(k); the last forward stage
-// pairs the addresses of k and k + N/2, which the spectrum needs together
-// with those of N - k and N/2 - k, so it is fused into the spectrum; the
-// spectrum's half-length sequence, left in the even addresses in
-// bit-reversed order, is what the decimation in time starts from.
-// What bounds it is the FP64 issue rate (two lanes per clock and SM): about
-// 6.8e5 FP64 instructions per level at N = 2^13.
-
-// Shared-memory slot of element i: bits 1-2 are XORed with bits 4-5, so that
-// the passes with a stride of two or eight elements spread over the banks.
-__device__ __forceinline__ int slot(int i) { return i ^ (((i >> 4) & 3) << 1); }
-
-__device__ __forceinline__ void bfly(double2& u, double2& v, double2 t) {
-  const double2 a = u;
-  u = make_double2(a.x + t.x, a.y + t.y);
-  v = make_double2(a.x - t.x, a.y - t.y);
-}
-
-// R stages s .. s + R - 1 of a transform of 2^lg values on the 2^R values
-// v[r] of one group; v[r] sits at position j + (r << s) within its block of
-// 2^(s + R) (positions as in fft_dit).  tw[k << tsh] = exp(-2 pi i k / 2^lg).
-template <int R, bool INV>
-__device__ __forceinline__ void group_stages(double2 (&v)[1 << R], const double2* tw, int lg,
-                                             int tsh, int s, int j) {
-#pragma unroll
-  for (int t = 0; t < R; ++t) {
-    const int sh = lg - 1 - s - t + tsh;
-#pragma unroll
-    for (int o = 0; o < (1 << t); ++o) {
-      const double2 w = tw[(j + (o << s)) << sh];
-#pragma unroll
-      for (int r = 0; r < (1 << R); r += 2 << t) {
-        const double2 b = v[r + o + (1 << t)];
-        bfly(v[r + o], v[r + o + (1 << t)], INV ? cmulc(w, b) : cmul(w, b));
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ int rev_bits(int k, int n) {
-  return n == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - n));
-}
-
-// Forward stages s .. s + R - 1 in place: the address of a position is its bit
-// reversal, so stage t pairs addresses that differ in bit lg - 1 - t.
-template <int R>
-__device__ __forceinline__ void fwd_pass(double2* a, const double2* tw, int lg, int s) {
-  const int low = lg - s - R;  // address bits below the group's
-  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
-    const int hi = g >> low, base = (hi << (low + R)) | (g & ((1 << low) - 1));
-    double2 v[1 << R];
-#pragma unroll
-    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(base + (rev_bits(r, R) << low))];
-    group_stages<R, false>(v, tw, lg, 0, s, rev_bits(hi, s));
-#pragma unroll
-    for (int r = 0; r < (1 << R); ++r) a[slot(base + (rev_bits(r, R) << low))] = v[r];
-  }
-  __syncthreads();
-}
-
-// Inverse stages s .. s + R - 1 of the 2^lg values in the even addresses.
-template <int R>
-__device__ __forceinline__ void inv_pass(double2* a, const double2* tw, int lg, int s) {
-  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
-    const int j = g & ((1 << s) - 1), base = ((g >> s) << (s + R)) | j;
-    double2 v[1 << R];
-#pragma unroll
-    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(2 * (base + (r << s)))];
-    group_stages<R, true>(v, tw, lg, 1, s, j);
-#pragma unroll
-    for (int r = 0; r < (1 << R); ++r) a[slot(2 * (base + (r << s)))] = v[r];
-  }
-  __syncthreads();
-}
-
 // First forward pass of R = 3 stages straight from the powered values: group j
 // holds the addresses j + t N / 8, of which t >= 4 are zero (n <= N / 2), so
 // stage 0 copies, stage 1 multiplies by 1 and -i, and half of stage 2 does.
@@ -859,55 +1253,14 @@ __device__ __forceinline__ void first_pass8(double2* a, const double2* tw, int l
 #pragma unroll
   for (int r = 0; r < 8; r += 4) {
     bfly(v[r], v[r + 2], v[r + 2]);
-    bfly(v[r + 1], v[r + 3], make_double2(v[r + 3].y, -v[r + 3].x));
+    bfly_mi(v[r + 1], v[r + 3]);
   }
   bfly(v[0], v[4], v[4]);
   bfly(v[1], v[5], cmul(tw[1 << (lg - 3)], v[5]));
-  bfly(v[2], v[6], make_double2(v[6].y, -v[6].x));
+  bfly_mi(v[2], v[6]);
   bfly(v[3], v[7], cmul(tw[3 << (lg - 3)], v[7]));
 #pragma unroll
   for (int r = 0; r < 8; ++r) a[slot(j + (rev_bits(r, 3) << (lg - 3)))] = v[r];
-}
-
-// The spectrum from the packed pair's transform (all but its last stage done)
-// to the half-length sequence 8 V_k in the even addresses; see conv_level.
-// The halves of the formulas there are left out: a power of two, exact.
-__device__ __forceinline__ void spectrum_pass(double2* a, const double2* tw, int lg) {
-  const int lm = lg - 1, M = 1 << lm;
-  for (int e = threadIdx.x; e <= (M >> 1); e += blockDim.x) {
-    // p = bitrev(k): 0, then the lower half of every [2^h, 2^(h + 1)); the
-    // address of M - k mirrors p within that range
-    int p = e, pm = e;
-    if (e > 1) {
-      const int f = e - 1, hb = 1 << (31 - __clz(f));
-      p = f + hb;
-      pm = p ^ (2 * hb - 1);
-    }
-    if (e > M >> 1 || p >= M) continue;
-    const int k = rev_bits(p, lm);
-    double2 ak = a[slot(2 * p)], amk = a[slot(2 * p + 1)];  // frequencies k, k + M
-    bfly(ak, amk, cmul(tw[k], amk));
-    double2 am = ak, an = amk;                              // M - k, N - k
-    if (k == 0) {
-      an = ak;  // N - 0 = 0 and M - 0 = M
-      am = amk;
-    } else if (pm != p) {
-      am = a[slot(2 * pm)];
-      an = a[slot(2 * pm + 1)];
-      bfly(am, an, cmul(tw[M - k], an));
-    }
-    auto z4 = [](double2 u, double2 v) {  // 4 spec_z
-      return cmul(make_double2(u.x + v.x, u.y - v.y), make_double2(u.y + v.y, -(u.x - v.x)));
-    };
-    auto v8 = [](double2 zk, double2 zm, double2 w) {  // 8 spec_v
-      const double2 o = cmulc(w, make_double2(zk.x - zm.x, zk.y + zm.y));
-      return make_double2((zk.x + zm.x) - o.y, (zk.y - zm.y) + o.x);
-    };
-    const double2 zk = z4(ak, an), zm = z4(am, amk);
-    a[slot(2 * p)] = v8(zk, zm, tw[k]);
-    if (k != 0 && pm != p) a[slot(2 * pm)] = v8(zm, zk, tw[M - k]);
-  }
-  __syncthreads();
 }
 
 // The p-sums.  Work items (problem, direction, level) in this order, each CTA
@@ -1016,14 +1369,7 @@ __global__ void __launch_bounds__(FFT_THREADS, 1)
       }
     }
     __syncthreads();
-    for (; s + 3 <= lg - 1; s += 3) fwd_pass<3>(a, tw, lg, s);
-    if (s + 2 == lg - 1) fwd_pass<2>(a, tw, lg, s);
-    else if (s + 1 == lg - 1) fwd_pass<1>(a, tw, lg, s);
-    spectrum_pass(a, tw, lg);
-    const int lm = lg - 1;
-    for (s = 0; s + 3 <= lm; s += 3) inv_pass<3>(a, tw, lm, s);
-    if (s + 2 == lm) inv_pass<2>(a, tw, lm, s);
-    else if (s + 1 == lm) inv_pass<1>(a, tw, lm, s);
+    conv_passes(a, tw, lg, s);
     const double scale = 0.25 / N;  // 2 / N, and the spectrum's 8
     double* sig = ta.sig + ((int64_t)pd * ta.n_p + q) * ta.nz;
     for (int m = tid; m < ta.nz; m += nt) {
@@ -1426,7 +1772,10 @@ int launch_maxconv_fft(const MaxconvArgs& ma, void* stream) {
   const cudaError_t e = cudaFuncSetAttribute(k_maxconv_fft,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_maxconv_fft<<<static_cast<unsigned>(ma.batch), FFT_THREADS, smem, s>>>(ma);
+  // eight values per thread: several CTAs per SM on short problems
+  const int N = 1 << ma.logN;
+  const int threads = N / 8 < 64 ? 64 : N / 8;
+  k_maxconv_fft<<<static_cast<unsigned>(ma.batch), threads, smem, s>>>(ma);
   return cudaGetLastError();
 }
 
