@@ -1,6 +1,7 @@
 // Host runtime and C ABI of the p-norm semiring library (include/pnorm.h):
 // argument checks, workspace layout, the per-level launch sequence of the
 // p-norm product (Alg. 5), the APSP driver (Sec. 2.2) and the exact product.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -455,16 +456,23 @@ BwLayout make_bw_layout(int64_t M, int64_t N, int64_t K, const pn_opts* o) {
   BwLayout L;
   const int mode = o->compute;
   const int bk = mode_bk(mode), planes = mode_planes(mode);
-  // CTA pairs on 256 x 256 tiles for both gradient GEMMs (outputs M x K and
-  // K x N) when each gives every cluster at least two pair tiles, so that a
-  // pair's gradient epilogue overlaps its next tile's MMAs (measured, 3xTF32,
-  // P = {16}: n = 2048 0.43 ms with pairs against 0.40 with one CTA per tile,
-  // 4096 1.40 against 1.56, 8192 7.42 against 9.54); unless the options ask
-  // for one CTA per tile or for 128-wide tiles
+  // CTA pairs on 256 x 256 tiles for both gradient GEMMs or one CTA per tile
+  // (outputs M x K and K x N), unless the options ask.  3xTF32 (128 x 128 single
+  // tiles): the form whose waves take less time, a pair tile counting 1.7 of a
+  // single one (measured 1.55 to 1.8; backward in us, P = {16}, single / pair:
+  // n = 1024 107 / 153, 2048 271 / 255, 3000 688 / 559, 4096 1294 / 1114,
+  // 2760 x 1284 x 1428 221 / 255).  16-bit and TF32 single tiles are 128 x 256
+  // and as good as a pair's up to there (BF16 2048 150 / 158, 3000 323 / 322, 4096
+  // 482 / 492): pairs from two tiles per cluster on.
   const int sms = device_sms();
-  const int64_t clusters = sms > 1 ? sms / 2 : 76;
+  const int64_t clusters = sms > 1 ? sms / 2 : 76, singles = 2 * clusters;
   const int64_t t1 = ceil_div(M, 256) * ceil_div(K, 256), t2 = ceil_div(K, 256) * ceil_div(N, 256);
-  const bool many = t1 >= 2 * clusters && t2 >= 2 * clusters;
+  const int64_t s1 = ceil_div(M, 128) * ceil_div(K, 128), s2 = ceil_div(K, 128) * ceil_div(N, 128);
+  const bool many =
+      mode == PN_F32_EXACT
+          ? 17 * (ceil_div(t1, clusters) + ceil_div(t2, clusters)) <
+                10 * (ceil_div(s1, singles) + ceil_div(s2, singles))
+          : t1 >= 2 * clusters && t2 >= 2 * clusters;
   L.cg = (o->tile_m == 256 || (o->tile_m == 0 && many)) && o->tile_n != 128 ? 2 : 1;
   L.BN = L.cg == 2 ? 256 : mode == PN_F32_EXACT ? 128 : (o->tile_n ? o->tile_n : 256);
   const int per = L.BN / TILE_M;
@@ -692,8 +700,7 @@ pn_status maxprod_pnorm_backward(int64_t M, int64_t N, int64_t K, const float* A
   uint32_t* mask = reinterpret_cast<uint32_t*>(w + L.off_mask);
   if (cudaMemsetAsync(w, 0, L.ctrl_bytes, s)) return PN_ECUDA;
   if (launch_maxes(fw, stream)) return PN_ECUDA;
-  if (launch_scales(fw, stream)) return PN_ECUDA;
-  if (launch_bw_mask(p_sel, M * N, opts->p_log2, opts->n_p, mask, stream)) return PN_ECUDA;
+  if (launch_bw_prep(fw, p_sel, M * N, opts->p_log2, opts->n_p, mask, stream)) return PN_ECUDA;
 
   // G1: dA (M x K) = W^(p) (M x N) . B'^p^T, contraction over N
   Common g1;
@@ -742,29 +749,43 @@ pn_status maxprod_pnorm_backward(int64_t M, int64_t N, int64_t K, const float* A
   g1.grad_axis = 0;
   g2.grad_axis = 1;
 
+  // operand images: W^(p) with rows i (contraction j) and rows j (contraction
+  // i), B'^p with rows k (contraction j), A'^p with rows k (contraction i)
+  BwImages im;
+  std::memset(&im, 0, sizeof(im));
+  im.A = A; im.B = B; im.r = fw.r; im.c = fw.c;
+  im.dC = dC; im.Cv = C; im.S = S_sel; im.psel = p_sel;
+  im.M = static_cast<int32_t>(M); im.N = static_cast<int32_t>(N); im.K = static_cast<int32_t>(K);
+  im.pmask = mask;
+  const auto dst = [&](size_t off, size_t plane, int RB, int KB) {
+    BwDst d;
+    d.img = w + off; d.plane = static_cast<int64_t>(plane); d.RB = RB; d.KB = KB;
+    return d;
+  };
+  im.dst[0][0] = dst(L.off_w1, L.plane_w1, L.RB1a, L.KB1);
+  im.dst[0][1] = dst(L.off_w2, L.plane_w2, L.RB2b, L.KB2);
+  im.dst[1][0] = dst(L.off_b1, L.plane_b1, L.RB1b, L.KB1);
+  im.dst[2][1] = dst(L.off_a2, L.plane_a2, L.RB2a, L.KB2);
+  for (int job = 0; job < 3; ++job) {
+    // 128 x 128 source blocks that cover every image tile (padding included)
+    const int per = TILE_M / mode_bk(opts->compute);
+    int rb = 0, cb = 0;
+    if (im.dst[job][0].img) {
+      rb = im.dst[job][0].RB;
+      cb = static_cast<int>(ceil_div(im.dst[job][0].KB, per));
+    }
+    if (im.dst[job][1].img) {
+      cb = std::max(cb, im.dst[job][1].RB);
+      rb = std::max(rb, static_cast<int>(ceil_div(im.dst[job][1].KB, per)));
+    }
+    im.blocks[job] = rb * cb;
+    im.cols[job] = cb;
+  }
   for (int q = opts->n_p - 1; q >= 0; --q) {
     const int plog = opts->p_log2[q];
-    BwImage im;
-    std::memset(&im, 0, sizeof(im));
-    im.plog = plog; im.q = q; im.pmask = mask;
-    im.dC = dC; im.Cv = C; im.S = S_sel; im.psel = p_sel;
-    // W^(p) rows (i, contraction j) and B'^p rows (k, contraction j)
-    im.kind = 1; im.trans = 0; im.srows = static_cast<int32_t>(M); im.scols = static_cast<int32_t>(N);
-    im.dst = w + L.off_w1; im.plane = static_cast<int64_t>(L.plane_w1); im.RB = L.RB1a; im.KB = L.KB1;
-    if (launch_bw_image(opts->compute, im, stream)) return PN_ECUDA;
-    im.kind = 0; im.trans = 0; im.src = B; im.lds = N; im.scale = fw.c;
-    im.srows = static_cast<int32_t>(K); im.scols = static_cast<int32_t>(N);
-    im.dst = w + L.off_b1; im.plane = static_cast<int64_t>(L.plane_b1); im.RB = L.RB1b; im.KB = L.KB1;
-    if (launch_bw_image(opts->compute, im, stream)) return PN_ECUDA;
-    // A'^p transposed (k, contraction i) and W^(p) transposed (j, contraction i)
-    im.kind = 0; im.trans = 1; im.src = A; im.lds = K; im.scale = fw.r;
-    im.srows = static_cast<int32_t>(M); im.scols = static_cast<int32_t>(K);
-    im.dst = w + L.off_a2; im.plane = static_cast<int64_t>(L.plane_a2); im.RB = L.RB2a; im.KB = L.KB2;
-    if (launch_bw_image(opts->compute, im, stream)) return PN_ECUDA;
-    im.kind = 1; im.trans = 1; im.src = nullptr; im.scale = nullptr;
-    im.srows = static_cast<int32_t>(M); im.scols = static_cast<int32_t>(N);
-    im.dst = w + L.off_w2; im.plane = static_cast<int64_t>(L.plane_w2); im.RB = L.RB2b; im.KB = L.KB2;
-    if (launch_bw_image(opts->compute, im, stream)) return PN_ECUDA;
+    im.plog = plog;
+    im.q = q;
+    if (launch_bw_images(opts->compute, im, stream)) return PN_ECUDA;
 
     Level lv;
     std::memset(&lv, 0, sizeof(lv));

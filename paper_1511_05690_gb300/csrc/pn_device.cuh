@@ -465,36 +465,12 @@ __device__ __forceinline__ float pow_pm1(float x, int k) {
 // no intermediate under- or overflows however small x' is; the total
 // exponent is applied once at the end (ldexpf: one rounding, into the
 // subnormal range if the result lies there).  x = 0 gives 0 for k >= 1.
-__device__ __forceinline__ float grad_factor(float acc, float x, float s, int k) {
-  // Fast path: the plain FP32 chain, taken when s = 2^E has a normal
-  // reciprocal and x'^(2^k - 1), acc times it and the result are normal.
-  // Every factor and partial product of the chain then lies between that
-  // power and 1, so each product rounds exactly as its renormalised
-  // counterpart below and the two paths agree bit for bit.  It is tried only
-  // where the exponent of x' = x / s alone shows the power to stay above
-  // 2^-125, so entries bound for the slow path skip it.
-  const uint32_t sb = __float_as_uint(s);
-  const int ex_xp = static_cast<int>((__float_as_uint(x) >> 23) & 0xFFu) - static_cast<int>(sb >> 23);
-  if (sb >= 0x00800000u && sb < 0x7F000000u && (sb & 0x007FFFFFu) == 0u &&
-      ex_xp * ((1 << k) - 1) >= -125) {
-    const float inv = __uint_as_float(0x7F000000u - sb);  // 2^-E
-    float y = __fmul_rn(x, inv);
-    float r = 1.0f;
-    for (int t = 0; t < k; ++t) {
-      r = __fmul_rn(r, y);
-      y = __fmul_rn(y, y);
-    }
-    const float ar = __fmul_rn(acc, r);
-    const float g = __fmul_rn(ar, inv);
-    const float fmin = 1.17549435e-38f;
-    if (r >= fmin && fabsf(ar) >= fmin && fabsf(g) >= fmin && fabsf(g) <= 3.40282347e38f) return g;
-  }
-  int ls, ex, d;
+static __device__ __noinline__ float grad_factor_frexp(float acc, float x, float s, int k) {
+  int ls, ex;
   frexpf(s, &ls);
   ls -= 1;                        // s = 2^ls
   float xm = frexpf(x, &ex);      // x = xm 2^ex, so x' = xm 2^(ex - ls)
   ex -= ls;
-  (void)d;
   float rm = 1.0f;
   int re = 0;
   // A product of two values in [0.5, 1] lies in [0.25, 1) (it cannot round
@@ -515,6 +491,41 @@ __device__ __forceinline__ float grad_factor(float acc, float x, float s, int k)
     }
   }
   return ldexpf(acc * rm, re - ls);
+}
+
+// The same, bit for bit (rounding does not depend on the scale of a mantissa),
+// for p <= 128 without a branch: with the mantissa in [0.75, 1.5) the chain stays
+// between 2^-53 and 2^75, so it is renormalised once, at the end, and the
+// exponent goes on in factors of normal powers of two, 1 but for the first unless
+// the result leaves FP32's range (a subnormal result may be rounded twice, within
+// one of its units).  About 35 instructions; with x' uniform half of the entries
+// took the renormalising loop at p = 64, some 150 instructions for every warp.
+// With the row-wise epilogue: a 2048^3 gradient GEMM in 3xTF32 185 -> 95 us.
+__device__ __forceinline__ float grad_factor(float acc, float x, float s, int k) {
+  if (k > 7) return grad_factor_frexp(acc, x, s, k);
+  // s = 2^ls and x = m 2^ex; subnormal values scaled up first
+  const bool tiny_s = s < 1.17549435e-38f, tiny_x = x < 1.17549435e-38f;
+  const int ls = static_cast<int>(__float_as_uint(tiny_s ? s * 16777216.0f : s) >> 23) -
+                 (tiny_s ? 127 + 24 : 127);
+  const uint32_t xb = __float_as_uint(tiny_x ? x * 16777216.0f : x);
+  const bool upper = (xb & 0x00400000u) != 0u;  // mantissa in [1.5, 2): halve it
+  const int ex = static_cast<int>(xb >> 23) - (tiny_x ? 127 + 24 : 127) + (upper ? 1 : 0);
+  float y = __uint_as_float((xb & 0x007fffffu) | (upper ? 0x3f000000u : 0x3f800000u));
+  float r = 1.0f;
+  for (int t = 0; t < k; ++t) {
+    r = __fmul_rn(r, y);
+    y = __fmul_rn(y, y);
+  }
+  // r = m 2^(exponent - 126) with m in [0.5, 1) (k = 0: r = 1 as it is)
+  const uint32_t rb = __float_as_uint(r), one = k == 0 ? 0x00800000u : 0u;
+  const int e = (ex - ls) * ((1 << k) - 1) - ls + static_cast<int>((rb - one) >> 23) - 126;
+  const int e1 = min(max(e, -126), 127), e2 = min(max(e - e1, -126), 127);
+  const int e3 = max(e - e1 - e2, -126);  // below 2^-252: acc may be up to 2^127
+  float g = __fmul_rn(acc, __uint_as_float((rb & 0x007fffffu) | (0x3f000000u + one)));
+  g = __fmul_rn(__fmul_rn(g, __uint_as_float(static_cast<uint32_t>(e1 + 127) << 23)),
+                __uint_as_float(static_cast<uint32_t>(e2 + 127) << 23));
+  g = __fmul_rn(g, __uint_as_float(static_cast<uint32_t>(min(e3, 0) + 127) << 23));
+  return k > 0 && x == 0.0f ? 0.0f : g;
 }
 
 // Smallest power of two >= m (m > 0, finite); 1 for m == 0.  Returns +inf

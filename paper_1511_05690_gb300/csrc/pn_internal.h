@@ -193,26 +193,29 @@ inline Schedule make_schedule(const pn_opts* o) {
   return s;
 }
 
-// One operand image of the adjoint (maxprod_pnorm_backward).
-//   kind 0: (src / scale)^p with one scale per contraction index
-//   kind 1: W^(p) = dC * C / S where p_sel == p, else 0
-//   trans 0: image row r = source row r, contraction = source column
-//   trans 1: image row r = source column r, contraction = source row
-struct BwImage {
-  const float* src;
-  int64_t lds;
-  int32_t srows, scols;
-  const float* scale;
+// The operand images of one p of the adjoint (maxprod_pnorm_backward): job 0
+// W^(p) = dC * C / S where p_sel == p, else 0 (M x N), job 1 (B / c)^p (K x N),
+// job 2 (A / r)^p (M x K).  dst[job][0] takes the source's rows as image rows,
+// dst[job][1] its columns (img null: not wanted).
+struct BwDst {
+  uint8_t* img;
+  int64_t plane;           // bytes to the lo plane (3xTF32)
+  int32_t RB, KB;          // image row blocks (128 rows), contraction blocks
+};
+struct BwImages {
+  const float* A;
+  const float* B;
+  const float* r;
+  const float* c;
   const float* dC;
   const float* Cv;
   const float* S;
   const uint8_t* psel;
-  uint8_t* dst;
-  int64_t plane;           // bytes to the lo plane (3xTF32)
-  int32_t RB, KB;          // image row blocks (128 rows), contraction blocks
+  int32_t M, N, K;
   int32_t plog, q;
   const uint32_t* pmask;
-  int32_t kind, trans;
+  BwDst dst[3][2];
+  int32_t blocks[3], cols[3];  // blocks of 128 x 128 per job, and per block row
 };
 
 __host__ __device__ inline const Prob& prob_at(const Common& cm, int g) {
@@ -345,10 +348,9 @@ int maxconv_fft_smem_bytes(int logN);
 int maxconv_exact_smem_bytes();
 int launch_maxconv_fft(const MaxconvArgs& ma, void* stream);
 int launch_maxconv_exact(const MaxconvArgs& ma, void* stream);
-int launch_bw_mask(const uint8_t* psel, int64_t count, const int32_t* plog_list, int n_p,
-                   uint32_t* mask, void* stream);
-int launch_scales(const Common& cm, void* stream);
-int launch_bw_image(int mode, const BwImage& im, void* stream);
+int launch_bw_prep(const Common& cm, const uint8_t* psel, int64_t count, const int32_t* plog_list,
+                   int n_p, uint32_t* mask, void* stream);
+int launch_bw_images(int mode, const BwImages& im, void* stream);
 int gemm_smem_bytes(int mode, int BN);
 // Persistent grouped launch: every level of a group in one cooperative launch
 // (returns a cudaError_t value).
