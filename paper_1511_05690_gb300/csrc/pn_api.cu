@@ -411,8 +411,7 @@ pn_status run_pnorm(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda
   const Schedule sc = make_schedule(o);
   for (int t = 0; t < sc.n; ++t) {
     const Level lv = make_level(L, o, ws, sc, t);
-    if ((e = launch_power_a(cm, lv, stream, &maps))) return PN_ECUDA;
-    if ((e = launch_power_b(cm, lv, stream, &maps))) return PN_ECUDA;
+    if ((e = launch_images(cm, lv, stream, &maps))) return PN_ECUDA;
     if (lv.is_top && o->correction == 2) {
       // the affine model's coefficients, from the scales of the top level
       FitArgs fa;

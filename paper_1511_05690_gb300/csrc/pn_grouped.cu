@@ -394,8 +394,7 @@ static pn_status run_group(const GroupHeader* H, const void* dev_table, int l, c
       if (lv.is_top && !top_inside && launch_strips(cm, lv, stream)) return PN_ECUDA;
       continue;
     }
-    if (launch_power_a(cm, lv, stream)) return PN_ECUDA;
-    if (launch_power_b(cm, lv, stream)) return PN_ECUDA;
+    if (launch_images(cm, lv, stream)) return PN_ECUDA;
     if (lv.is_top && o->ev_gemm_begin)
       if (cudaEventRecord(static_cast<cudaEvent_t>(o->ev_gemm_begin), s)) return PN_ECUDA;
     if (launch_gemm_level(cm, lv, sms, stream)) return PN_ECUDA;

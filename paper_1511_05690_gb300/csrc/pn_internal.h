@@ -312,10 +312,9 @@ int launch_maxes(const Common& cm, void* stream);
 // Grouped top level (scaling 0 or 2): maxima, domain test, scales and images
 // of every operand block in one launch (a CTA per 32-row / 32-column strip).
 int launch_strips(const Common& cm, const Level& lv, void* stream);
-int launch_power_a(const Common& cm, const Level& lv, void* stream,
-                   const OperandMaps* maps = nullptr);
-int launch_power_b(const Common& cm, const Level& lv, void* stream,
-                   const OperandMaps* maps = nullptr);
+// The level's powered operand images of A and B.
+int launch_images(const Common& cm, const Level& lv, void* stream,
+                  const OperandMaps* maps = nullptr);
 int launch_gemm_level(const Common& cm, const Level& lv, int num_sms, void* stream);
 int launch_fused(const Common& cm, const FusedArgs& fa, void* stream);
 int launch_exact(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,

@@ -189,13 +189,13 @@ __global__ void __launch_bounds__(PRO_THREADS) k_maxes(const __grid_constant__ C
 // and the block then builds the flagged ones in order.  `needed(id)` and
 // `body(id)` must be block-uniform in effect (body may synchronise the block).
 template <typename Need, typename Body>
-__device__ __forceinline__ void for_flagged_ids(int total, const Need& needed, const Body& body) {
+__device__ __forceinline__ void for_flagged_ids(int bid, int grid, int total, const Need& needed, const Body& body) {
   __shared__ uint32_t mask[PRO_THREADS / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_ids = blockIdx.x < total ? (total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int n_ids = bid < total ? (total - 1 - bid) / grid + 1 : 0;
   for (int j0 = 0; j0 < n_ids; j0 += PRO_THREADS) {
     const int j = j0 + threadIdx.x;
-    const bool need = j < n_ids && needed((int)blockIdx.x + j * (int)gridDim.x);
+    const bool need = j < n_ids && needed(bid + j * grid);
     const uint32_t b = __ballot_sync(0xffffffffu, need);
     if (lane == 0) mask[warp] = b;
     __syncthreads();
@@ -204,7 +204,7 @@ __device__ __forceinline__ void for_flagged_ids(int total, const Need& needed, c
       while (m) {
         const int bit = __ffs(m) - 1;
         m &= m - 1;
-        body((int)blockIdx.x + (j0 + w * 32 + bit) * (int)gridDim.x);
+        body(bid + (j0 + w * 32 + bit) * grid);
       }
     }
     __syncthreads();  // mask is rewritten by the next round
@@ -217,12 +217,9 @@ constexpr int img_min_blocks() {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
-    k_power_a(const __grid_constant__ Common cm, const __grid_constant__ Level lv) {
-  pdl_wait();
-  pdl_trigger();
+__device__ __forceinline__ void power_a_blocks(const Common& cm, const Level& lv, int bid, int grid) {
   if (lv.is_top) {
-    const int id = blockIdx.x;
+    const int id = bid;
     const int g = find_prob(cm, id, 1);
     const Prob& P = prob_at(cm, g);
     const int local = id - P.xa_base;
@@ -232,7 +229,7 @@ __global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
   }
   if (*lv.work_count == 0) return;  // no tile pushed to this level (uniform)
   for_flagged_ids(
-      cm.total_xa,
+      bid, grid, cm.total_xa,
       [&](int id) {
         const Prob& P = prob_at(cm, find_prob(cm, id, 1));
         return lv.rflag[P.tm_base + (id - P.xa_base) / P.KB] != 0;
@@ -250,13 +247,10 @@ __global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
 // as for A, a tile is rebuilt only if a pushed output tile needs its tile
 // column.
 template <int MODE>
-__global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
-    k_power_b(const __grid_constant__ Common cm, const __grid_constant__ Level lv) {
-  extern __shared__ float stile[];  // [BK][129]
-  pdl_wait();
-  pdl_trigger();
+__device__ __forceinline__ void power_b_blocks(const Common& cm, const Level& lv, float* stile,
+                                               int bid, int grid) {
   if (lv.is_top) {
-    const int id = blockIdx.x;
+    const int id = bid;
     const int g = find_prob(cm, id, 2);
     const Prob& P = prob_at(cm, g);
     const int local = id - P.xb_base;
@@ -267,7 +261,7 @@ __global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
   if (*lv.work_count == 0) return;  // no tile pushed to this level (uniform)
   const int per_tile = cm.BN / TILE_M;
   for_flagged_ids(
-      cm.total_xb,
+      bid, grid, cm.total_xb,
       [&](int id) {
         const Prob& P = prob_at(cm, find_prob(cm, id, 2));
         return lv.cflag[P.tn_base + (id - P.xb_base) / P.KB / per_tile] != 0;
@@ -279,6 +273,21 @@ __global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
         const int rb = local / P.KB;
         power_b_tile<MODE>(cm, lv, g, P, rb, local - rb * P.KB, stile, threadIdx.x, 0);
       });
+}
+
+// Both operands' per-tile images in one launch: blocks 0 .. n_a - 1 take A, the
+// others B.
+template <int MODE>
+__global__ void __launch_bounds__(PRO_THREADS, img_min_blocks<MODE>())
+    k_power(const __grid_constant__ Common cm, const __grid_constant__ Level lv, int n_a) {
+  extern __shared__ float stile[];  // [BK][129] (B)
+  pdl_wait();
+  pdl_trigger();
+  const int bid = blockIdx.x;
+  if (bid < n_a)
+    power_a_blocks<MODE>(cm, lv, bid, n_a);
+  else
+    power_b_blocks<MODE>(cm, lv, stile, bid - n_a, gridDim.x - n_a);
 }
 
 // ------------------------------------------------ TMA top-level images ---
@@ -343,12 +352,13 @@ __device__ __forceinline__ void lds_rotated(const float* src, int rot, float* v)
   }
 }
 
+// The images of one operand by CTA `bid` of `grid` (see the kernels below);
+// tile_k[MAX_OWNED] and n_tiles are shared memory, one copy for both operands
+// (a second copy left room for one CTA per SM instead of two: 712 against
+// 485 us at n = 16384 in bf16).
 template <int MODE, bool IS_B>
-__global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B>::CTAS)
-    k_image_tma(const __grid_constant__ Common cm, const __grid_constant__ Level lv,
-                const __grid_constant__ CUtensorMap map) {
-  pdl_wait();
-  pdl_trigger();
+__device__ __forceinline__ void image_tma(const Common& cm, const Level& lv, const CUtensorMap& map,
+                                          int bid, int grid, int32_t* tile_k, int32_t& n_tiles) {
   using CF = TmaCfg<MODE, IS_B>;
   using PK = Packer<MODE>;
   constexpr int EPC = PK::EPC;
@@ -365,14 +375,12 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Prob& P = cm.single;
   const int total = IS_B ? cm.total_xb : cm.total_xa;
-  const int owned = (int)blockIdx.x < total ? (total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int owned = bid < total ? (total - 1 - bid) / grid + 1 : 0;
   if (owned == 0) return;  // uniform
   if (!lv.is_top && *lv.work_count == 0) return;  // no tile pushed to this level (uniform)
-  // This CTA's tiles: ids blockIdx.x + k * gridDim.x, k < owned; below the top
+  // This CTA's tiles: ids bid + k * grid, k < owned; below the top
   // level only those whose row block (A) or tile column (B) is flagged,
   // compacted into tile_k[] (the launcher bounds owned by CF::MAX_OWNED).
-  __shared__ int32_t tile_k[CF::MAX_OWNED];
-  __shared__ int32_t n_tiles;
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
     *abort_flag = 0;
@@ -389,7 +397,7 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
       const int k = k0 + tid;
       bool need = false;
       if (k < owned) {
-        const int rb = ((int)blockIdx.x + k * (int)gridDim.x) / P.KB;
+        const int rb = (bid + k * grid) / P.KB;
         need = IS_B ? lv.cflag[rb / per_tile] != 0 : lv.rflag[rb] != 0;
       }
       const uint32_t bal = __ballot_sync(0xffffffffu, need);
@@ -407,7 +415,7 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
   // thread 0: the tensor copy of this CTA's j-th stage (tile j / H, half
   // j % H of its K values) into ring slot j % NST
   auto issue = [&](int j) {
-    const int id = (int)blockIdx.x + tile_k[j / H] * (int)gridDim.x;
+    const int id = bid + tile_k[j / H] * grid;
     const int rb = id / P.KB, kb = id - rb * P.KB;
     const int k0 = kb * BK + (j % H) * SBK;
     uint64_t* bar = &full[j % NST];
@@ -440,7 +448,7 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
   // j, loaded one tile ahead of their use
   uint32_t pre[U];
   auto prefetch = [&](int jj) {
-    const int rbj = ((int)blockIdx.x + tile_k[jj] * (int)gridDim.x) / P.KB;
+    const int rbj = (bid + tile_k[jj] * grid) / P.KB;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int idx = rbj * TILE_M + line(u);
@@ -468,7 +476,7 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
     __syncthreads();  // also: the shared B image ((j / H) & 1) is free again
     if (*abort_flag) break;
     const int tj = j / H, h = j % H;
-    const int id = (int)blockIdx.x + tile_k[tj] * (int)gridDim.x;
+    const int id = bid + tile_k[tj] * grid;
     const int rb = id / P.KB, kb = id - rb * P.KB;
     const int cc = ccl + CPR * h;  // this thread's chunk of the image row
     const float* st = ring + s * (CF::STAGE_BYTES / 4);
@@ -530,6 +538,29 @@ __global__ void __launch_bounds__(TmaCfg<MODE, IS_B>::THREADS, TmaCfg<MODE, IS_B
     }
     if constexpr (IS_B) bulk_wait_all();
   }
+}
+
+// Both operands in one launch (a level's launches cost about 3 us of host time
+// and 1.3 us on the GPU each, also where the level has nothing to do): the
+// first n_a CTAs take A, the others B.  One launch against two, every level:
+// 112.7 against 122 us for the whole 1021 x 2047 x 1531 product in bf16, 790
+// against 820 us at n = 4096 with estimator 1; at n = 16384 the top level's
+// images take 485 us, 231 + 262 us apart.
+template <int MODE>
+__global__ void __launch_bounds__(TmaCfg<MODE, true>::THREADS, TmaCfg<MODE, true>::CTAS)
+    k_image_tma(const __grid_constant__ Common cm, const __grid_constant__ Level lv,
+                const __grid_constant__ CUtensorMap map_a,
+                const __grid_constant__ CUtensorMap map_b, int n_a) {
+  static_assert(TmaCfg<MODE, false>::THREADS == TmaCfg<MODE, true>::THREADS, "one block size");
+  pdl_wait();
+  pdl_trigger();
+  __shared__ int32_t tile_k[TmaCfg<MODE, true>::MAX_OWNED];
+  __shared__ int32_t n_tiles;
+  const int bid = blockIdx.x;
+  if (bid < n_a)
+    image_tma<MODE, false>(cm, lv, map_a, bid, n_a, tile_k, n_tiles);
+  else
+    image_tma<MODE, true>(cm, lv, map_b, bid - n_a, gridDim.x - n_a, tile_k, n_tiles);
 }
 
 // ------------------------------------------------------------ K == 0 ---
@@ -603,34 +634,43 @@ int sm_count() {
   return sms;
 }
 
-template <int MODE, bool IS_B>
-int launch_tma_t(const Common& cm, const Level& lv, void* stream, const TensorMapBytes& map) {
-  using CF = TmaCfg<MODE, IS_B>;
+template <int MODE>
+int launch_tma_t(const Common& cm, const Level& lv, void* stream, const OperandMaps& maps, int xa,
+                 int xb) {
+  using CA = TmaCfg<MODE, false>;
+  using CB = TmaCfg<MODE, true>;
+  constexpr int smem = CA::SMEM > CB::SMEM ? CA::SMEM : CB::SMEM;
   static bool attr_done = false;
   if (!attr_done) {
     const cudaError_t e = cudaFuncSetAttribute(
-        k_image_tma<MODE, IS_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, CF::SMEM);
+        k_image_tma<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  const int total = IS_B ? cm.total_xb : cm.total_xa;
-  const int grid = total < CF::CTAS * sm_count() ? total : CF::CTAS * sm_count();
-  const cudaError_t e = launch_pdl(k_image_tma<MODE, IS_B>, dim3(grid), dim3(CF::THREADS), CF::SMEM,
-                                   stream, cm, lv, *reinterpret_cast<const CUtensorMap*>(&map));
+  // the resident CTAs, shared out by the operands' tiles
+  const int total = xa + xb;
+  const int grid = total < CB::CTAS * sm_count() ? total : CB::CTAS * sm_count();
+  int n_a = xb == 0 ? grid : static_cast<int>(static_cast<int64_t>(grid) * xa / total);
+  if (xa > 0 && n_a == 0) n_a = 1;
+  if (xb > 0 && n_a == grid) n_a = grid - 1;
+  const cudaError_t e = launch_pdl(k_image_tma<MODE>, dim3(grid), dim3(CB::THREADS), smem, stream, cm,
+                                   lv, *reinterpret_cast<const CUtensorMap*>(&maps.a),
+                                   *reinterpret_cast<const CUtensorMap*>(&maps.b), n_a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // The tensor-copy kernel takes at most TMA_MAX_OWNED tiles per SM.
 bool tma_fits(int total) { return total <= TMA_MAX_OWNED * sm_count(); }
 
-template <bool IS_B>
-int launch_tma(const Common& cm, const Level& lv, void* stream, const TensorMapBytes& map) {
+// xa / xb: tiles of A / B to build (0: not this operand).
+int launch_tma(const Common& cm, const Level& lv, void* stream, const OperandMaps& maps, int xa,
+               int xb) {
   switch (cm.mode) {
-    case MODE_3XTF32: return launch_tma_t<MODE_3XTF32, IS_B>(cm, lv, stream, map);
-    case MODE_TF32: return launch_tma_t<MODE_TF32, IS_B>(cm, lv, stream, map);
-    case MODE_BF16: return launch_tma_t<MODE_BF16, IS_B>(cm, lv, stream, map);
-    case MODE_F16: return launch_tma_t<MODE_F16, IS_B>(cm, lv, stream, map);
-    case MODE_E4M3: return launch_tma_t<MODE_E4M3, IS_B>(cm, lv, stream, map);
+    case MODE_3XTF32: return launch_tma_t<MODE_3XTF32>(cm, lv, stream, maps, xa, xb);
+    case MODE_TF32: return launch_tma_t<MODE_TF32>(cm, lv, stream, maps, xa, xb);
+    case MODE_BF16: return launch_tma_t<MODE_BF16>(cm, lv, stream, maps, xa, xb);
+    case MODE_F16: return launch_tma_t<MODE_F16>(cm, lv, stream, maps, xa, xb);
+    case MODE_E4M3: return launch_tma_t<MODE_E4M3>(cm, lv, stream, maps, xa, xb);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -676,18 +716,31 @@ bool encode_fp32_2d(TensorMapBytes& out, const float* base, int64_t rows, int64_
 }
 
 template <int MODE>
-int launch_power_b_t(const Common& cm, const Level& lv, void* stream) {
-  const int smem = mode_bk(MODE) * 129 * 4;
+int launch_power_t(const Common& cm, const Level& lv, void* stream, int xa, int xb) {
+  const int smem = xb > 0 ? mode_bk(MODE) * 129 * 4 : 0;
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_power_b<MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_power<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, mode_bk(MODE) * 129 * 4);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  const int grid = lv.is_top ? cm.total_xb : lower_grid(cm.total_xb, img_min_blocks<MODE>());
-  const cudaError_t e = launch_pdl(k_power_b<MODE>, dim3(grid), dim3(PRO_THREADS), smem, stream, cm, lv);
+  const int n_a = lv.is_top ? xa : lower_grid(xa, img_min_blocks<MODE>());
+  const int n_b = lv.is_top ? xb : lower_grid(xb, img_min_blocks<MODE>());
+  const cudaError_t e =
+      launch_pdl(k_power<MODE>, dim3(n_a + n_b), dim3(PRO_THREADS), smem, stream, cm, lv, n_a);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+int launch_power(const Common& cm, const Level& lv, void* stream, int xa, int xb) {
+  switch (cm.mode) {
+    case MODE_3XTF32: return launch_power_t<MODE_3XTF32>(cm, lv, stream, xa, xb);
+    case MODE_TF32: return launch_power_t<MODE_TF32>(cm, lv, stream, xa, xb);
+    case MODE_BF16: return launch_power_t<MODE_BF16>(cm, lv, stream, xa, xb);
+    case MODE_F16: return launch_power_t<MODE_F16>(cm, lv, stream, xa, xb);
+    case MODE_E4M3: return launch_power_t<MODE_E4M3>(cm, lv, stream, xa, xb);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 int grid_for(int64_t total, int threads) {
@@ -1004,48 +1057,17 @@ void make_operand_maps(const Common& cm, OperandMaps& maps) {
   maps.has_b = encode_fp32_2d(maps.b, P.B, P.K, P.N, P.ldb, bk, TILE_M) ? 1 : 0;
 }
 
-int launch_power_a(const Common& cm, const Level& lv, void* stream, const OperandMaps* maps) {
-  if (cm.total_xa <= 0) return 0;
-  if (maps && maps->has_a && tma_fits(cm.total_xa)) return launch_tma<false>(cm, lv, stream, maps->a);
-  auto grid = [&](int per_sm) { return lv.is_top ? cm.total_xa : lower_grid(cm.total_xa, per_sm); };
-  cudaError_t e = cudaSuccess;
-  switch (cm.mode) {
-    case MODE_3XTF32:
-      e = launch_pdl(k_power_a<MODE_3XTF32>, dim3(grid(img_min_blocks<MODE_3XTF32>())), dim3(PRO_THREADS), 0,
-                     stream, cm, lv);
-      break;
-    case MODE_TF32:
-      e = launch_pdl(k_power_a<MODE_TF32>, dim3(grid(img_min_blocks<MODE_TF32>())), dim3(PRO_THREADS), 0,
-                     stream, cm, lv);
-      break;
-    case MODE_BF16:
-      e = launch_pdl(k_power_a<MODE_BF16>, dim3(grid(img_min_blocks<MODE_BF16>())), dim3(PRO_THREADS), 0,
-                     stream, cm, lv);
-      break;
-    case MODE_F16:
-      e = launch_pdl(k_power_a<MODE_F16>, dim3(grid(img_min_blocks<MODE_F16>())), dim3(PRO_THREADS), 0,
-                     stream, cm, lv);
-      break;
-    case MODE_E4M3:
-      e = launch_pdl(k_power_a<MODE_E4M3>, dim3(grid(img_min_blocks<MODE_E4M3>())), dim3(PRO_THREADS), 0,
-                     stream, cm, lv);
-      break;
-    default: return cudaErrorInvalidValue;
-  }
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-int launch_power_b(const Common& cm, const Level& lv, void* stream, const OperandMaps* maps) {
-  if (cm.total_xb <= 0) return 0;
-  if (maps && maps->has_b && tma_fits(cm.total_xb)) return launch_tma<true>(cm, lv, stream, maps->b);
-  switch (cm.mode) {
-    case MODE_3XTF32: return launch_power_b_t<MODE_3XTF32>(cm, lv, stream);
-    case MODE_TF32: return launch_power_b_t<MODE_TF32>(cm, lv, stream);
-    case MODE_BF16: return launch_power_b_t<MODE_BF16>(cm, lv, stream);
-    case MODE_F16: return launch_power_b_t<MODE_F16>(cm, lv, stream);
-    case MODE_E4M3: return launch_power_b_t<MODE_E4M3>(cm, lv, stream);
-    default: return cudaErrorInvalidValue;
-  }
+int launch_images(const Common& cm, const Level& lv, void* stream, const OperandMaps* maps) {
+  const int xa = cm.total_xa, xb = cm.total_xb;
+  const bool ta = maps && maps->has_a && tma_fits(xa), tb = maps && maps->has_b && tma_fits(xb);
+  int e = 0;
+  if (ta && tb && tma_fits(xa + xb))
+    return xa + xb > 0 ? launch_tma(cm, lv, stream, *maps, xa, xb) : 0;
+  if (ta && xa > 0) e = launch_tma(cm, lv, stream, *maps, xa, 0);
+  if (!e && tb && xb > 0) e = launch_tma(cm, lv, stream, *maps, 0, xb);
+  const int pa = ta ? 0 : xa, pb = tb ? 0 : xb;
+  if (!e && pa + pb > 0) e = launch_power(cm, lv, stream, pa, pb);
+  return e;
 }
 
 int launch_fill_empty(const Common& cm, int plog0, void* stream) {
