@@ -109,8 +109,12 @@ __device__ void fft_dit(double2* a, const double2* tw, int logL, int tws) {
 // (S)^(1/2^plog): plog correctly rounded FP32 square roots of float(S) for
 // S >= 1e-30 (the output is FP32; relative error about (plog + 1) 2^-24),
 // FP64 square roots below that (only unstable indices at the smallest p).
+// (Compared as integers: positive values order alike, and no FP64 slot is taken.)
+__device__ __forceinline__ bool ge_pos(double v, double bound) {  // bound > 0, v no NaN
+  return __double_as_longlong(v) >= __double_as_longlong(bound);
+}
 __device__ __forceinline__ double root_pow2(double S, int plog) {
-  if (S >= 1e-30) {
+  if (ge_pos(S, 1e-30)) {
     float r = static_cast<float>(S);
     for (int s = 0; s < plog; ++s) r = sqrtf(r);
     return r;
@@ -166,28 +170,6 @@ __device__ void direct_levels(const MaxconvArgs& ma, const float* x, const float
   }
   z[m] = static_cast<float>(sxy * root_pow2(s_sel, ma.p_log2[qs]));
   res[m] = static_cast<uint8_t>(ma.p_log2[qs] | (stable ? 0 : 0x80));
-}
-
-// In-place radix-2 decimation-in-frequency FFT of a[0..L) in natural order;
-// bit-reversed order on return; unscaled; INV: conjugate twiddles.
-template <bool INV>
-__device__ void fft_dif(double2* a, const double2* tw, int logL, int tws) {
-  const int L = 1 << logL;
-  for (int s = logL - 1; s >= 0; --s) {
-    const int h = 1 << s;
-    const int step = ((L >> 1) >> s) * tws;
-    for (int b = threadIdx.x; b < (L >> 1); b += static_cast<int>(blockDim.x)) {
-      const int j = b & (h - 1);
-      const int i0 = ((b >> s) << (s + 1)) + j;
-      const int i1 = i0 + h;
-      const double2 u = a[i0], v = a[i1];
-      const double2 d = make_double2(u.x - v.x, u.y - v.y);
-      a[i0] = make_double2(u.x + v.x, u.y + v.y);
-      const double2 w = tw[j * step];
-      a[i1] = INV ? cmulc(w, d) : cmul(w, d);
-    }
-    __syncthreads();
-  }
 }
 
 // Z_k from A_k and A_(N-k) (the spectra of the packed real pair).
@@ -399,12 +381,36 @@ __device__ __forceinline__ void bfly(C& u, C& v, C t) {
   v = c_sub(a, t);
 }
 
-// The butterfly with the twiddle -i.  (A negated FP64 value costs an FP64
-// instruction unless it is the subtrahend of the operation that uses it.)
+// The butterfly with the twiddle -i (INV: +i).  (A negated FP64 value costs an
+// FP64 instruction unless it is the subtrahend of the operation that uses it.)
+template <bool INV = false>
 __device__ __forceinline__ void bfly_mi(double2& u, double2& v) {
   const double2 a = u, b = v;
-  u = make_double2(a.x + b.y, a.y - b.x);
-  v = make_double2(a.x - b.y, a.y + b.x);
+  const double2 p = make_double2(a.x + b.y, a.y - b.x), m = make_double2(a.x - b.y, a.y + b.x);
+  u = INV ? m : p;
+  v = INV ? p : m;
+}
+
+// Stages 0 to 2 of a transform on the 8 values of positions 0..7 of a block,
+// w1 and w3 = exp(-2 pi i / 8), exp(-6 pi i / 8) as tabled: the twiddles 1 and
+// -+i take no product (their products are exact).  HALF: the values of odd
+// positions, the upper half of the input, are zero and not read.
+template <bool INV, bool HALF>
+__device__ __forceinline__ void first_stages8(double2 (&v)[8], double2 w1, double2 w3) {
+#pragma unroll
+  for (int r = 0; r < 8; r += 2) {
+    if constexpr (HALF) v[r + 1] = v[r];
+    else bfly(v[r], v[r + 1], v[r + 1]);
+  }
+#pragma unroll
+  for (int r = 0; r < 8; r += 4) {
+    bfly(v[r], v[r + 2], v[r + 2]);
+    bfly_mi<INV>(v[r + 1], v[r + 3]);
+  }
+  bfly(v[0], v[4], v[4]);
+  bfly(v[1], v[5], INV ? cmulc(w1, v[5]) : cmul(w1, v[5]));
+  bfly_mi<INV>(v[2], v[6]);
+  bfly(v[3], v[7], INV ? cmulc(w3, v[7]) : cmul(w3, v[7]));
 }
 
 // R stages s .. s + R - 1 of a transform of 2^lg values on the 2^R values
@@ -432,17 +438,18 @@ __device__ __forceinline__ int rev_bits(int k, int n) {
   return n == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - n));
 }
 
-// Forward stages s .. s + R - 1 in place: the address of a position is its bit
-// reversal, so stage t pairs addresses that differ in bit lg - 1 - t.
-template <int R, typename C>
-__device__ __forceinline__ void fwd_pass(C* a, const C* tw, int lg, int s) {
+// Stages s .. s + R - 1 in place, by threads t of nt: the address of a position
+// is its bit reversal, so stage t pairs addresses that differ in bit lg - 1 - t.
+template <int R, bool INV = false, typename C>
+__device__ __forceinline__ void fwd_pass(C* a, const C* tw, int lg, int s, int t = threadIdx.x,
+                                         int nt = blockDim.x) {
   const int low = lg - s - R;  // address bits below the group's
-  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+  for (int g = t; g < (1 << (lg - R)); g += nt) {
     const int hi = g >> low, base = (hi << (low + R)) | (g & ((1 << low) - 1));
     C v[1 << R];
 #pragma unroll
     for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(base + (rev_bits(r, R) << low))];
-    group_stages<R, false>(v, tw, lg, 0, s, rev_bits(hi, s));
+    group_stages<R, INV>(v, tw, lg, 0, s, rev_bits(hi, s));
 #pragma unroll
     for (int r = 0; r < (1 << R); ++r) a[slot(base + (rev_bits(r, R) << low))] = v[r];
   }
@@ -937,12 +944,25 @@ __global__ void __launch_bounds__(MCX_THREADS)
 //   forward  A[k1 + N1 k2] = sum_n2 W_N2^(n2 k2) [W_N^(n2 k1) sum_n1 a[n] W_N1^(n1 k1)]
 //   inverse  s[n] = sum_k1 W_N1^-(n1 k1) [W_N^-(n2 k1) sum_k2 Z[k1 + N1 k2] W_N2^-(n2 k2)]
 // Three kernels per level: columns forward (the powered inputs are formed on
-// the fly), row pairs (forward rows, spectrum, inverse rows: row k1 holds the
-// partners N - k of row N1 - k1), columns inverse with the selection.  A
+// the fly), rows (forward row, spectrum, inverse row; row k1 holds the
+// partners N - k of row N1 - k1, so two CTAs of a cluster take these two rows
+// and read each other's spectrum), columns inverse with the selection.  A
 // fourth kernel ends the level loop (nothing open) or sums the remaining
 // levels directly for few open terms.  All kernels of a finished call return
 // at once (device flag), so every launch is issued unconditionally.
-constexpr int LONG_CC = 8;   // columns per CTA of the column kernels
+//
+// The transforms are radix-2 butterflies in FP64 throughout (the values near
+// tau at the edges carry their rounding, and p_sel depends on it), eight values
+// per thread in registers for three stages; the first and last three stages
+// read from and write to global memory.  What bounds them is the FP64 rate,
+// two lanes per clock and SM: 7.5e8 instructions at N = 2^22, 1.3 ms.  Hence
+// no products with 1 and -+i, no first stage where the upper half of the input
+// is zero, two CTAs per SM to fill each other's barriers, and pieces small
+// enough for a full last wave (1024 of each kind on 152 SMs, 6.7 per SM, against 512
+// in 3.4 waves).  n = 2^21 per vector: 1538 us per call (column kernels about 315 each, rows 815), 2160 with a barrier
+// per stage, 8 columns or a pair of rows per CTA.
+constexpr int LONG_CC = 4;   // columns per CTA of the column kernels
+constexpr int LONG_THREADS = 512;
 
 struct LongArgs {
   const float* x;
@@ -959,7 +979,7 @@ struct LongArgs {
   const double2* tlo;      // W_N^m, m < 2048
   const double2* thi;      // W_N^(2048 m), m < N / 2048
   unsigned long long* open_terms;  // per level
-  int32_t* done;
+  int32_t* done;                   // 0; 1 + the level that was the last; -1 on bad input
   uint32_t* mxy;           // max x, max y (float bits)
 };
 
@@ -967,37 +987,41 @@ __device__ __forceinline__ double2 w_n(const LongArgs& la, int m) {
   return cmul(la.thi[m >> 11], la.tlo[m & 2047]);
 }
 
-__global__ void k_long_tables(double2* tlo, double2* thi, int logN) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const double N = static_cast<double>(1 << logN);
-  double s, c;
-  if (k < 2048) {
-    sincospi(-2.0 * k / N, &s, &c);
-    tlo[k] = make_double2(c, s);
-  }
-  if (k < ((1 << logN) >> 11)) {
-    sincospi(-2.0 * (2048.0 * k) / N, &s, &c);
-    thi[k] = make_double2(c, s);
-  }
-}
+constexpr int LONG_TAB_BLOCKS = 8, LONG_MAX_BLOCKS = 152 * 4;  // of 256 threads
 
-__global__ void k_long_max(const __grid_constant__ LongArgs la) {
+// The tables of W_N^m (the first blocks), the maxima and the domain test (the rest).
+__global__ void k_long_init(const __grid_constant__ LongArgs la, double2* tlo, double2* thi) {
+  if (blockIdx.x < LONG_TAB_BLOCKS) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const double N = static_cast<double>(1 << la.logN);
+    double s, c;
+    if (k < 2048) {
+      sincospi(-2.0 * k / N, &s, &c);
+      tlo[k] = make_double2(c, s);
+    }
+    if (k < ((1 << la.logN) >> 11)) {
+      sincospi(-2.0 * (2048.0 * k) / N, &s, &c);
+      thi[k] = make_double2(c, s);
+    }
+    return;
+  }
+  const int first = (blockIdx.x - LONG_TAB_BLOCKS) * blockDim.x + threadIdx.x;
   float mx = 0.0f, my = 0.0f;
   bool bad = false;
-  const int stride = gridDim.x * blockDim.x;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < la.nx; k += stride) {
+  const int stride = LONG_MAX_BLOCKS * blockDim.x;
+  for (int k = first; k < la.nx; k += stride) {
     const float v = la.x[k];
     bad |= !(v >= 0.0f && v <= 3.4028235e38f);
     mx = fmaxf(mx, v);
   }
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < la.ny; k += stride) {
+  for (int k = first; k < la.ny; k += stride) {
     const float v = la.y[k];
     bad |= !(v >= 0.0f && v <= 3.4028235e38f);
     my = fmaxf(my, v);
   }
   if (bad) {
     set_status(la.status, PN_EDOMAIN);
-    *la.done = 1;  // nothing more runs
+    *la.done = -1;  // nothing more runs
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -1017,125 +1041,314 @@ __device__ __forceinline__ void long_scales(const LongArgs& la, double& sx, doub
   if (sy == 0.0) sy = 1.0;
 }
 
+// Elements between the columns in shared memory: columns of the same address
+// two slots apart.
+__device__ __forceinline__ int long_col_stride(int l1) { return (1 << l1) + 2; }
+
+__device__ __forceinline__ void long_twiddles(double2* tw, int lg) {
+  for (int k = threadIdx.x; k < (1 << (lg - 1)); k += blockDim.x)
+    tw[k] = g_twiddle[k << (FFT_LOG_NMAX - lg)];
+}
+
+// Stages 3 .. lg - 4 of a transform whose first three stages are done.
+template <bool INV>
+__device__ __forceinline__ void long_middle(double2* a, const double2* tw, int lg, int t, int nt) {
+  int s = 3;
+  const int end = lg - 3;
+  while (s < end) {
+    if (end - s == 3 || end - s >= 5) {
+      fwd_pass<3, INV>(a, tw, lg, s, t, nt);
+      s += 3;
+    } else if (end - s >= 2) {
+      fwd_pass<2, INV>(a, tw, lg, s, t, nt);
+      s += 2;
+    } else {
+      fwd_pass<1, INV>(a, tw, lg, s, t, nt);
+      s += 1;
+    }
+  }
+}
+
 // columns [c0, c0 + CC): a[N2 n1 + n2] = x'^p + i y'^p, DFT over n1 (length
-// N1), times W_N^(n2 k1), stored row-major as buf[k1 N2 + n2].
-__global__ void __launch_bounds__(FFT_THREADS, 1)
+// N1), times W_N^(n2 k1), stored row-major as buf[k1 N2 + n2].  CC N1 / 8 threads.
+__global__ void __launch_bounds__(LONG_THREADS, 2)
     k_long_col_fwd(const __grid_constant__ LongArgs la, int q) {
+  pdl_wait();
+  pdl_trigger();
   if (*la.done) return;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N1 = 1 << la.l1, N2 = 1 << la.l2;
-  double2* col = reinterpret_cast<double2*>(smem);   // [CC][N1]
-  double2* tw = col + LONG_CC * N1;                   // N1 / 2
-  const int tid = threadIdx.x;
-  for (int k = tid; k < (N1 >> 1); k += FFT_THREADS) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - la.l1)];
-  double sx, sy;
-  long_scales(la, sx, sy);
-  const float isx = static_cast<float>(1.0 / sx), isy = static_cast<float>(1.0 / sy);
+  __shared__ float inv[2];
+  const int l1 = la.l1, N1 = 1 << l1, N2 = 1 << la.l2;
+  const int tid = threadIdx.x, c = tid & (LONG_CC - 1), g = tid / LONG_CC, ng = N1 >> 3;
+  double2* col = reinterpret_cast<double2*>(smem);   // [CC][stride]
+  double2* tw = col + LONG_CC * long_col_stride(l1);  // N1 / 2
+  col += c * long_col_stride(l1);
+  long_twiddles(tw, l1);
+  if (tid == 0) {
+    double sx, sy;
+    long_scales(la, sx, sy);
+    inv[0] = static_cast<float>(1.0 / sx);
+    inv[1] = static_cast<float>(1.0 / sy);
+  }
+  const int n2 = blockIdx.x * LONG_CC + c;
+  // v[r]: position r of the first three stages, n1 = g + rev3(r) N1 / 8
+  float xr[8], yr[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int n = (g + rev_bits(r, 3) * ng) * N2 + n2;
+    xr[r] = n < la.nx ? __ldg(la.x + n) : 0.0f;
+    yr[r] = n < la.ny ? __ldg(la.y + n) : 0.0f;
+  }
+  __syncthreads();
+  const float isx = inv[0], isy = inv[1];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    xr[r] *= isx;
+    yr[r] *= isy;
+  }
   const int plog = la.p_log2[q];
-  const int c0 = blockIdx.x * LONG_CC;
-  for (int e = tid; e < LONG_CC * N1; e += FFT_THREADS) {
-    const int n1 = e / LONG_CC, c = e % LONG_CC;
-    const int n = n1 * N2 + c0 + c;
-    float xr = 0.0f, yr = 0.0f;
-    if (n < la.nx) {
-      xr = la.x[n] * isx;
-      for (int s = 0; s < plog; ++s) xr *= xr;
+#pragma unroll 1
+  for (int s = 0; s < plog; ++s) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      xr[r] *= xr[r];
+      yr[r] *= yr[r];
     }
-    if (n < la.ny) {
-      yr = la.y[n] * isy;
-      for (int s = 0; s < plog; ++s) yr *= yr;
+  }
+  double2 v[8];
+  if (max(la.nx, la.ny) <= (1 << (la.logN - 1))) {
+#pragma unroll
+    for (int r = 0; r < 8; r += 2) v[r] = make_double2(xr[r], yr[r]);
+    first_stages8<false, true>(v, tw[ng], tw[3 * ng]);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = make_double2(xr[r], yr[r]);
+    first_stages8<false, false>(v, tw[ng], tw[3 * ng]);
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) col[slot(g + rev_bits(r, 3) * ng)] = v[r];
+  __syncthreads();
+  long_middle<false>(col, tw, l1, g, ng);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) v[r] = col[slot(8 * g + rev_bits(r, 3))];
+  const int rg = rev_bits(g, l1 - 3);
+  group_stages<3, false>(v, tw, l1, 0, l1 - 3, rg);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int k1 = r * ng + rg;
+    la.buf[(int64_t)k1 * N2 + n2] = cmul(w_n(la, n2 * k1), v[r]);
+  }
+}
+
+// 4 spec_z(a, b), the halves left out (powers of two, exact).
+__device__ __forceinline__ double2 spec_z4(double2 a, double2 b) {
+  const double2 s = make_double2(a.x + b.x, a.y - b.y);
+  const double dy = a.y + b.y, ndx = b.x - a.x;  // -i (a - conj b) = (dy, ndx)
+  return make_double2(fma(s.x, dy, -__dmul_rn(s.y, ndx)), fma(s.x, ndx, __dmul_rn(s.y, dy)));
+}
+
+// R decimation-in-frequency stages of the inverse transform, in the natural
+// order of the addresses: position k sits at address bitrev(k), stage s = lg - 1
+// - b pairs addresses that differ in bit b; the result of address n is sample
+// n.  v[r] is at address (hi << (b0 + R)) + (r << b0) + any lower bits.
+template <int R>
+__device__ __forceinline__ void dif_stages(double2 (&v)[1 << R], const double2* tw, int lg, int b0,
+                                           int hi) {
+  const int nh = lg - b0 - R, rh = rev_bits(hi, nh);
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+#pragma unroll
+    for (int o = 0; o < (1 << (R - 1 - t)); ++o) {
+      const double2 w = tw[(rh + (rev_bits(o, R - 1 - t) << nh)) << (b0 + t)];
+#pragma unroll
+      for (int l = 0; l < (1 << t); ++l) {
+        const int r = (o << (t + 1)) + l, u = r + (1 << t);
+        const double2 d = c_sub(v[r], v[u]);
+        v[r] = c_add(v[r], v[u]);
+        v[u] = cmulc(w, d);
+      }
     }
-    col[c * N1 + bitrev(n1, la.l1)] = make_double2(xr, yr);
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void dif_pass(double2* a, const double2* tw, int lg, int b0) {
+  for (int g = threadIdx.x; g < (1 << (lg - R)); g += blockDim.x) {
+    const int hi = g >> b0, base = (hi << (b0 + R)) | (g & ((1 << b0) - 1));
+    double2 v[1 << R];
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) v[r] = a[slot(base + (r << b0))];
+    dif_stages<R>(v, tw, lg, b0, hi);
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) a[slot(base + (r << b0))] = v[r];
   }
   __syncthreads();
-  for (int c = 0; c < LONG_CC; ++c) fft_dit<false>(col + c * N1, tw, la.l1, 1);
-  for (int e = tid; e < LONG_CC * N1; e += FFT_THREADS) {
-    const int k1 = e / LONG_CC, c = e % LONG_CC;
-    const int n2 = c0 + c;
-    la.buf[(int64_t)k1 * N2 + n2] = cmul(w_n(la, n2 * k1), col[c * N1 + k1]);
-  }
 }
 
-// Z from a spectrum value and its partner (the packed real pair).
-__device__ __forceinline__ void pair_z(double2& a, double2& b) {
-  const double2 za = spec_z(a, b), zb = spec_z(b, a);
-  a = za;
-  b = zb;
+// The last three of them (twiddles as in first_stages8): v[u] becomes i (v[r] -
+// v[u]) or the plain difference where the twiddle is conj(-i) or 1.
+__device__ __forceinline__ void dif_last8(double2 (&v)[8], double2 w1, double2 w3) {
+  auto one = [&](int r, int u) {
+    const double2 d = c_sub(v[r], v[u]);
+    v[r] = c_add(v[r], v[u]);
+    v[u] = d;
+  };
+  auto by_i = [&](int r, int u) {
+    const double2 d = make_double2(v[u].y - v[r].y, v[r].x - v[u].x);
+    v[r] = c_add(v[r], v[u]);
+    v[u] = d;
+  };
+  one(0, 1);
+  by_i(2, 3);
+  one(4, 5);
+  v[5] = cmulc(w1, v[5]);
+  one(6, 7);
+  v[7] = cmulc(w3, v[7]);
+  one(0, 2);
+  one(1, 3);
+  by_i(4, 6);
+  by_i(5, 7);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) one(r, r + 4);
 }
 
-// rows k1 and N1 - k1 (blockIdx.x = k1 in [0, N1/2]; rows 0 and N1/2 alone)
-__global__ void __launch_bounds__(FFT_THREADS, 1)
+__device__ __forceinline__ double2 ld_cluster(uint32_t addr) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr));
+  return v;
+}
+
+// Rows k1 and N1 - k1 by the two CTAs of cluster k1 (cluster 0: the rows 0 and
+// N1 / 2, each its own partner), N2 / 8 threads (a warp at least).
+__global__ void __launch_bounds__(LONG_THREADS, 2)
     k_long_rows(const __grid_constant__ LongArgs la) {
+  pdl_wait();
+  pdl_trigger();
   if (*la.done) return;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N1 = 1 << la.l1, N2 = 1 << la.l2;
-  double2* r0 = reinterpret_cast<double2*>(smem);  // row k1
-  double2* r1 = r0 + N2;                            // row N1 - k1
-  double2* tw = r1 + N2;                            // N2 / 2
-  const int tid = threadIdx.x;
-  const int k1 = blockIdx.x, k1b = N1 - k1;
-  const bool two = k1 != 0 && k1 != (N1 >> 1);
-  for (int k = tid; k < (N2 >> 1); k += FFT_THREADS) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - la.l2)];
-  for (int k = tid; k < N2; k += FFT_THREADS) {
-    r0[bitrev(k, la.l2)] = la.buf[(int64_t)k1 * N2 + k];
-    if (two) r1[bitrev(k, la.l2)] = la.buf[(int64_t)k1b * N2 + k];
+  const int l2 = la.l2, N1 = 1 << la.l1, N2 = 1 << l2;
+  double2* a = reinterpret_cast<double2*>(smem);  // the row
+  double2* tw = a + N2;                            // N2 / 2
+  const int g = threadIdx.x, ng = N2 >> 3;
+  const uint32_t rank = cluster_ctarank();
+  const int id = static_cast<int>(cluster_id_x());
+  const int k1 = rank == 0 ? id : id == 0 ? N1 >> 1 : N1 - id;
+  double2* row = la.buf + (int64_t)k1 * N2;
+  long_twiddles(tw, l2);
+  double2 v[8];
+  if (g < ng) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = row[g + rev_bits(r, 3) * ng];
   }
   __syncthreads();
-  fft_dit<false>(r0, tw, la.l2, 1);
-  if (two) fft_dit<false>(r1, tw, la.l2, 1);
-  // spectrum in place: the partner of (k1, k2) is (N1 - k1, N2 - 1 - k2),
-  // of (0, k2) it is (0, (N2 - k2) mod N2)
-  if (two) {
-    for (int k2 = tid; k2 < N2; k2 += FFT_THREADS) pair_z(r0[k2], r1[N2 - 1 - k2]);
-  } else if (k1 == 0) {
-    for (int k2 = tid; k2 <= (N2 >> 1); k2 += FFT_THREADS) {
-      const int p2 = (N2 - k2) & (N2 - 1);
-      if (p2 == k2) r0[k2] = spec_z(r0[k2], r0[k2]);
-      else pair_z(r0[k2], r0[p2]);
+  if (g < ng) {
+    first_stages8<false, false>(v, tw[ng], tw[3 * ng]);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[slot(g + rev_bits(r, 3) * ng)] = v[r];
+  }
+  __syncthreads();
+  long_middle<false>(a, tw, l2, threadIdx.x, blockDim.x);
+  if (g < ng) {  // the last three stages; the values stay in registers too
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = a[slot(8 * g + rev_bits(r, 3))];
+    group_stages<3, false>(v, tw, l2, 0, l2 - 3, rev_bits(g, l2 - 3));
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[slot(8 * g + rev_bits(r, 3))] = v[r];
+  }
+  __syncwarp();
+  cluster_sync_all();
+  // the spectrum: frequency k2 is at address bitrev(k2); the partner of
+  // (k1, k2) is (N1 - k1, N2 - 1 - k2), the complement of the address, of (0, k2)
+  // it is (0, (N2 - k2) mod N2)
+  double2 z[8];  // by address 8 g + r
+  if (g < ng) {
+    const uint32_t peer = mapa_shared(smem_u32(a), id == 0 ? rank : rank ^ 1u);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int at = 8 * g + r;
+      const int pa = k1 == 0 ? rev_bits((N2 - rev_bits(at, l2)) & (N2 - 1), l2) : N2 - 1 - at;
+      z[r] = spec_z4(v[rev_bits(r, 3)], ld_cluster(peer + 16u * static_cast<uint32_t>(slot(pa))));
     }
-  } else {
-    for (int k2 = tid; k2 < (N2 >> 1); k2 += FFT_THREADS) pair_z(r0[k2], r0[N2 - 1 - k2]);
+  }
+  __syncwarp();
+  cluster_sync_all();  // both rows are read
+  if (g < ng) {
+    dif_stages<3>(z, tw, l2, 0, g);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[slot(8 * g + r)] = z[r];
   }
   __syncthreads();
-  fft_dif<true>(r0, tw, la.l2, 1);
-  if (two) fft_dif<true>(r1, tw, la.l2, 1);
-  // bit-reversed rows; times conj W_N^(n2 k1)
-  for (int n2 = tid; n2 < N2; n2 += FFT_THREADS) {
-    la.buf[(int64_t)k1 * N2 + n2] = cmulc(w_n(la, n2 * k1), r0[bitrev(n2, la.l2)]);
-    if (two) la.buf[(int64_t)k1b * N2 + n2] = cmulc(w_n(la, n2 * k1b), r1[bitrev(n2, la.l2)]);
+  int b0 = 3;
+  const int end = l2 - 3;
+  while (b0 < end) {
+    if (end - b0 == 3 || end - b0 >= 5) {
+      dif_pass<3>(a, tw, l2, b0);
+      b0 += 3;
+    } else if (end - b0 >= 2) {
+      dif_pass<2>(a, tw, l2, b0);
+      b0 += 2;
+    } else {
+      dif_pass<1>(a, tw, l2, b0);
+      b0 += 1;
+    }
+  }
+  if (g < ng) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) z[r] = a[slot(g + r * ng)];
+    dif_last8(z, tw[ng], tw[3 * ng]);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int n2 = g + r * ng;
+      row[n2] = cmulc(w_n(la, n2 * k1), z[r]);
+    }
   }
 }
 
-// columns [c0, c0 + CC): inverse DFT over k1 gives s[N2 n1 + n2]; the
+// columns [c0, c0 + CC): inverse DFT over k1 gives 4 s[N2 n1 + n2]; the
 // selection of level q for every open index; open terms counted for the
 // direct-sum decision.
-__global__ void __launch_bounds__(FFT_THREADS, 1)
+__global__ void __launch_bounds__(LONG_THREADS, 2)
     k_long_col_inv(const __grid_constant__ LongArgs la, int q) {
+  pdl_wait();
+  pdl_trigger();
   if (*la.done) return;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N1 = 1 << la.l1, N2 = 1 << la.l2;
+  __shared__ double scale;
+  const int l1 = la.l1, N1 = 1 << l1, N2 = 1 << la.l2;
+  const int tid = threadIdx.x, c = tid & (LONG_CC - 1), g = tid / LONG_CC, ng = N1 >> 3;
   double2* col = reinterpret_cast<double2*>(smem);
-  double2* tw = col + LONG_CC * N1;
-  const int tid = threadIdx.x;
-  for (int k = tid; k < (N1 >> 1); k += FFT_THREADS) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - la.l1)];
-  const int c0 = blockIdx.x * LONG_CC;
-  for (int e = tid; e < LONG_CC * N1; e += FFT_THREADS) {
-    const int k1 = e / LONG_CC, c = e % LONG_CC;
-    col[c * N1 + bitrev(k1, la.l1)] = la.buf[(int64_t)k1 * N2 + c0 + c];
+  double2* tw = col + LONG_CC * long_col_stride(l1);
+  col += c * long_col_stride(l1);
+  long_twiddles(tw, l1);
+  if (tid == 0) {
+    double sx, sy;
+    long_scales(la, sx, sy);
+    scale = sx * sy;
   }
+  const int n2 = blockIdx.x * LONG_CC + c;
+  double2 v[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) v[r] = la.buf[(int64_t)(g + rev_bits(r, 3) * ng) * N2 + n2];
   __syncthreads();
-  for (int c = 0; c < LONG_CC; ++c) fft_dit<true>(col + c * N1, tw, la.l1, 1);
-  double sx, sy;
-  long_scales(la, sx, sy);
-  const double sxy = sx * sy, invN = 1.0 / static_cast<double>(1 << la.logN);
+  first_stages8<true, false>(v, tw[ng], tw[3 * ng]);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) col[slot(g + rev_bits(r, 3) * ng)] = v[r];
+  __syncthreads();
+  long_middle<true>(col, tw, l1, g, ng);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) v[r] = col[slot(8 * g + rev_bits(r, 3))];
+  const int rg = rev_bits(g, l1 - 3);
+  group_stages<3, true>(v, tw, l1, 0, l1 - 3, rg);
+  const double sxy = scale;
+  const double inv4n = __hiloint2double((1023 - 2 - la.logN) << 20, 0);  // 1 / (4 N)
   const int plog = la.p_log2[q];
   unsigned long long terms = 0ull;
-  for (int e = tid; e < LONG_CC * N1; e += FFT_THREADS) {
-    const int n1 = e / LONG_CC, c = e % LONG_CC;
-    const int m = n1 * N2 + c0 + c;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int m = (r * ng + rg) * N2 + n2;
     if (m >= la.nz || la.res[m] != 0xFF) continue;
-    const double S = col[c * N1 + n1].x * invN;
-    const bool stable = S >= la.tau;
+    const double S = v[r].x * inv4n;
+    const bool stable = ge_pos(S, la.tau);
     if (stable || q == 0) {
       la.z[m] = static_cast<float>(sxy * root_pow2(S, plog));
       la.res[m] = static_cast<uint8_t>(plog | (stable ? 0 : 0x80));
@@ -1150,11 +1363,14 @@ __global__ void __launch_bounds__(FFT_THREADS, 1)
 // directly for every remaining level (then the call ends); otherwise the
 // next level runs.
 __global__ void k_long_direct(const __grid_constant__ LongArgs la, int q) {
-  if (*la.done) return;
+  pdl_wait();
+  pdl_trigger();
+  const int done = *la.done;  // may already be this level's, by block 0
+  if (done != 0 && done != q + 1) return;
   const unsigned long long W = la.open_terms[q];
   const int N = 1 << la.logN;
   if (W == 0ull || q == 0) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *la.done = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *la.done = q + 1;
     return;
   }
   if (W * static_cast<unsigned long long>(8 + 2 * q) >
@@ -1171,7 +1387,7 @@ __global__ void k_long_direct(const __grid_constant__ LongArgs la, int q) {
   const double isy = static_cast<double>(static_cast<float>(1.0 / sy));
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < la.nz; m += gridDim.x * blockDim.x)
     if (la.res[m] == 0xFF) direct_levels(ma, la.x, la.y, isx, isy, sx * sy, m, q, la.z, la.res);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *la.done = 1;  // read by the next launches only
+  if (blockIdx.x == 0 && threadIdx.x == 0) *la.done = q + 1;
 }
 
 // ------------------------------------------------------------ top-k x y ---
@@ -1248,17 +1464,9 @@ __device__ __forceinline__ void first_pass8(double2* a, const double2* tw, int l
 #pragma unroll
   for (int r = 0; r < 8; r += 2) {
     const int t = ((r >> 1) & 1) * 2 + (r >> 2);  // rev3(r), r even
-    v[r] = v[r + 1] = make_double2(x[t], y[t]);
+    v[r] = make_double2(x[t], y[t]);
   }
-#pragma unroll
-  for (int r = 0; r < 8; r += 4) {
-    bfly(v[r], v[r + 2], v[r + 2]);
-    bfly_mi(v[r + 1], v[r + 3]);
-  }
-  bfly(v[0], v[4], v[4]);
-  bfly(v[1], v[5], cmul(tw[1 << (lg - 3)], v[5]));
-  bfly_mi(v[2], v[6]);
-  bfly(v[3], v[7], cmul(tw[3 << (lg - 3)], v[7]));
+  first_stages8<false, true>(v, tw[1 << (lg - 3)], tw[3 << (lg - 3)]);
 #pragma unroll
   for (int r = 0; r < 8; ++r) a[slot(j + (rev_bits(r, 3) << (lg - 3)))] = v[r];
 }
@@ -1855,23 +2063,38 @@ int launch_maxconv_long(const pn_opts* o, int64_t nx, const float* x, int64_t ny
   la.mxy = reinterpret_cast<uint32_t*>(ws + L.off_ctrl + 136);
   if ((e = cudaMemsetAsync(ws + L.off_ctrl, 0, 256, s))) return e;
   if ((e = cudaMemsetAsync(la.res, 0xFF, static_cast<size_t>(nz), s))) return e;
-  k_long_tables<<<8, 256, 0, s>>>(reinterpret_cast<double2*>(ws + L.off_tlo),
-                                  reinterpret_cast<double2*>(ws + L.off_thi), la.logN);
-  k_long_max<<<152 * 4, 256, 0, s>>>(la);
+  k_long_init<<<LONG_TAB_BLOCKS + LONG_MAX_BLOCKS, 256, 0, s>>>(
+      la, reinterpret_cast<double2*>(ws + L.off_tlo), reinterpret_cast<double2*>(ws + L.off_thi));
+  if ((e = cudaGetLastError())) return e;
   const int N1 = 1 << la.l1, N2 = 1 << la.l2;
-  const int smem_col = (LONG_CC * N1 + N1 / 2) * static_cast<int>(sizeof(double2));
-  const int smem_row = (2 * N2 + N2 / 2) * static_cast<int>(sizeof(double2));
+  const int smem_col = (LONG_CC * (N1 + 2) + N1 / 2) * static_cast<int>(sizeof(double2));
+  const int smem_row = (N2 + N2 / 2) * static_cast<int>(sizeof(double2));
   if ((e = cudaFuncSetAttribute(k_long_col_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col)))
     return e;
   if ((e = cudaFuncSetAttribute(k_long_col_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col)))
     return e;
   if ((e = cudaFuncSetAttribute(k_long_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_row)))
     return e;
+  const dim3 cols(N2 / LONG_CC), col_threads(LONG_CC * N1 / 8);
+  cudaLaunchConfig_t rows = {};
+  rows.gridDim = dim3(N1);
+  rows.blockDim = dim3(N2 / 8 < 32 ? 32 : N2 / 8);
+  rows.dynamicSmemBytes = smem_row;
+  rows.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_pdl
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  rows.attrs = attr;
+  rows.numAttrs = 2;
   for (int q = o->n_p - 1; q >= 0; --q) {
-    k_long_col_fwd<<<N2 / LONG_CC, FFT_THREADS, smem_col, s>>>(la, q);
-    k_long_rows<<<N1 / 2 + 1, FFT_THREADS, smem_row, s>>>(la);
-    k_long_col_inv<<<N2 / LONG_CC, FFT_THREADS, smem_col, s>>>(la, q);
-    k_long_direct<<<152 * 4, 256, 0, s>>>(la, q);
+    if ((e = launch_pdl(k_long_col_fwd, cols, col_threads, smem_col, s, la, q))) return e;
+    if ((e = cudaLaunchKernelEx(&rows, k_long_rows, la))) return e;
+    if ((e = launch_pdl(k_long_col_inv, cols, col_threads, smem_col, s, la, q))) return e;
+    if ((e = launch_pdl(k_long_direct, dim3(152 * 4), dim3(256), 0, s, la, q))) return e;
   }
   return cudaGetLastError();
 }
