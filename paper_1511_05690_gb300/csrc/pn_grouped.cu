@@ -315,6 +315,9 @@ static pn_status run_group(const GroupHeader* H, const void* dev_table, int l, c
   for (int w = 0; w < 7; ++w)
     cm.lut[w] = reinterpret_cast<const int32_t*>(static_cast<const uint8_t*>(dev_table) + L.lut_offset[w]);
   cm.nprob = H->count;
+  // the kernels take a lone problem's record from the arguments (prob_at)
+  if (H->count == 1)
+    std::memcpy(&cm.single, reinterpret_cast<const uint8_t*>(H) + L.probs_offset, sizeof(Prob));
   cm.total_tiles = L.total_tiles;
   cm.total_xa = L.total_xa;
   cm.total_xb = L.total_xb;
