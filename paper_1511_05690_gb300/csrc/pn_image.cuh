@@ -108,22 +108,33 @@ __device__ __forceinline__ void div_scales(float (&v)[U][EPC], const float (&s)[
 
 // v <- v^p * opscale with p = 2^plog, or p = 1.5 * 2^plog for a half level
 // (y * sqrt(y), y = v^(2^plog)); the squarings of all U x EPC values
-// interleaved (independent chains; the same products as pow2k value by value).
+// interleaved (independent chains; the same products as pow2k value by value),
+// two per instruction: the strips of grouped products run out of issue slots.
 template <int U, int EPC>
 __device__ __forceinline__ void power_all(float (&v)[U][EPC], int plog, int half, float opscale) {
+  uint64_t w[U][EPC / 2];  // two values per instruction
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int e = 0; e < EPC; e += 2) w[u][e / 2] = f32x2_pack(v[u][e], v[u][e + 1]);
 #pragma unroll 1
   for (int t = 0; t < plog; ++t) {
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int e = 0; e < EPC; ++e) v[u][e] *= v[u][e];
+      for (int e = 0; e < EPC / 2; ++e) w[u][e] = f32x2_mul(w[u][e], w[u][e]);
   }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int e = 0; e < EPC; e += 2) f32x2_unpack(w[u][e / 2], v[u][e], v[u][e + 1]);
   if (half) {
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int e = 0; e < EPC; ++e) v[u][e] *= sqrtf(v[u][e]);
   }
+  if (opscale == 1.0f) return;
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
