@@ -179,6 +179,13 @@ __device__ __forceinline__ double2 spec_z(double2 ak, double2 an) {
   return cmul(X, Y);
 }
 
+// 4 spec_z(a, b), the halves left out (powers of two, exact).
+__device__ __forceinline__ double2 spec_z4(double2 a, double2 b) {
+  const double2 s = make_double2(a.x + b.x, a.y - b.y);
+  const double dy = a.y + b.y, ndx = b.x - a.x;  // -i (a - conj b) = (dy, ndx)
+  return make_double2(fma(s.x, dy, -__dmul_rn(s.y, ndx)), fma(s.x, ndx, __dmul_rn(s.y, dy)));
+}
+
 // V_k = (Z_k + conj Z_(M-k)) / 2 + i conj(W^k) (Z_k - conj Z_(M-k)) / 2, w = W^k.
 __device__ __forceinline__ double2 spec_v(double2 zk, double2 zmk, double2 w) {
   const double2 e = make_double2(0.5 * (zk.x + zmk.x), 0.5 * (zk.y - zmk.y));
@@ -332,7 +339,6 @@ __device__ __forceinline__ double2 c_sub_conj(double2 a, double2 b) {
 __device__ __forceinline__ double2 c_add_i(double2 a, double2 b) {
   return make_double2(a.x - b.y, a.y + b.x);
 }
-__device__ __forceinline__ double2 c_mul_mi(double2 a) { return make_double2(a.y, -a.x); }
 __device__ __forceinline__ cff c_add(cff a, cff b) { return ff_add(a.h, a.l, b.h, b.l); }
 __device__ __forceinline__ cff c_sub(cff a, cff b) { return ff_sub(a.h, a.l, b.h, b.l); }
 __device__ __forceinline__ cff c_conj(cff a) {
@@ -471,6 +477,20 @@ __device__ __forceinline__ void inv_pass(C* a, const C* tw, int lg, int s) {
   __syncthreads();
 }
 
+// Inverse stages 0 to 2 (first_stages8), FP64.
+__device__ __forceinline__ void inv_first_pass(double2* a, const double2* tw, int lg) {
+  const double2 w1 = tw[2 << (lg - 3)], w3 = tw[6 << (lg - 3)];
+  for (int g = threadIdx.x; g < (1 << (lg - 3)); g += blockDim.x) {
+    double2 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = a[slot(2 * (8 * g + r))];
+    first_stages8<true, false>(v, w1, w3);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[slot(2 * (8 * g + r))] = v[r];
+  }
+  __syncthreads();
+}
+
 // The spectrum from the packed pair's transform (all but its last stage done)
 // to the half-length sequence 8 V_k in the even addresses; see conv_level.
 // The halves of the formulas there are left out: a power of two, exact.
@@ -500,7 +520,8 @@ __device__ __forceinline__ void spectrum_pass(C* a, const C* tw, int lg) {
       bfly(am, an, cmul(tw_at(tw, M - k), an));
     }
     auto z4 = [](C u, C v) {  // 4 spec_z: (u + conj v) (-i (u - conj v))
-      return cmul(c_add_conj(u, v), c_mul_mi(c_sub_conj(u, v)));
+      if constexpr (std::is_same_v<C, double2>) return spec_z4(u, v);
+      else return cmul(c_add_conj(u, v), c_mul_mi(c_sub_conj(u, v)));
     };
     auto v8 = [](C zk, C zm, C w) {  // 8 spec_v
       return c_add_i(c_add_conj(zk, zm), cmulc(w, c_sub_conj(zk, zm)));
@@ -524,7 +545,12 @@ __device__ __forceinline__ void conv_passes(double2* a, const double2* tw, int l
   else if (s + 1 == lg - 1) fwd_pass<1>(a, tw, lg, s);
   spectrum_pass(a, tw, lg);
   const int lm = lg - 1;
-  for (s = 0; s + 3 <= lm; s += 3) inv_pass<3>(a, tw, lm, s);
+  s = 0;
+  if (lm >= 3) {
+    inv_first_pass(a, tw, lm);
+    s = 3;
+  }
+  for (; s + 3 <= lm; s += 3) inv_pass<3>(a, tw, lm, s);
   if (s + 2 == lm) inv_pass<2>(a, tw, lm, s);
   else if (s + 1 == lm) inv_pass<1>(a, tw, lm, s);
 }
@@ -1138,13 +1164,6 @@ __global__ void __launch_bounds__(LONG_THREADS, 2)
     const int k1 = r * ng + rg;
     la.buf[(int64_t)k1 * N2 + n2] = cmul(w_n(la, n2 * k1), v[r]);
   }
-}
-
-// 4 spec_z(a, b), the halves left out (powers of two, exact).
-__device__ __forceinline__ double2 spec_z4(double2 a, double2 b) {
-  const double2 s = make_double2(a.x + b.x, a.y - b.y);
-  const double dy = a.y + b.y, ndx = b.x - a.x;  // -i (a - conj b) = (dy, ndx)
-  return make_double2(fma(s.x, dy, -__dmul_rn(s.y, ndx)), fma(s.x, ndx, __dmul_rn(s.y, dy)));
 }
 
 // R decimation-in-frequency stages of the inverse transform, in the natural
