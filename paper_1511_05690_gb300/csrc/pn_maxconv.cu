@@ -1495,7 +1495,7 @@ __device__ __forceinline__ void first_pass8(double2* a, const double2* tw, int l
 // problem and direction ran 512 pairs of the 256-problem batch as 3.37 waves
 // of 152, the last one mostly empty), and the values x'^p, y'^p of a pair stay
 // in registers and are squared from level to level.
-// 256 problems of n = 4096, 13 levels: 8.24 ms (12.29 ms with one CTA per
+// 256 problems of n = 4096, 13 levels: 7.99 ms (12.29 ms with one CTA per
 // problem and direction and two stages per pass).
 __global__ void __launch_bounds__(FFT_THREADS, 1)
     k_topk_sums(const __grid_constant__ TopkArgs ta) {
