@@ -195,8 +195,8 @@ pn_status pn_grouped_build_table(int32_t count, const int64_t* MNK, const float*
   // order: the persistent kernel's CTA c takes the tiles c, c + SMs, ..., so the
   // long contractions spread evenly and the last tiles are the cheapest, and
   // the longest strips of the image kernel start first (64 problems of 16 to
-  // 1024 in BF16: 42.3 us for the persistent kernel and 35.1 for the strips,
-  // 44.4 and 38.7 in the caller's order).
+  // 1024 in BF16: 42.3 us for the persistent kernel and 36.3 for the strips,
+  // 44.4 and 38.5 in the caller's order).
   std::vector<int32_t> order(static_cast<size_t>(count));
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),

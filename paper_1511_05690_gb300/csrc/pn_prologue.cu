@@ -759,10 +759,11 @@ int grid_for(int64_t total, int threads) {
 // power_b_tile (same scales, same operation order), so the images are
 // bit-identical to theirs.  What bounds a strip is instruction issue (57 % of the
 // slots) and the latency of its loads: the scale's reciprocal and the check
-// for it are taken once, rows and columns past the operand are only zeroed, two
-// squarings go in an instruction and the next k-block's loads are issued before
-// this one's arithmetic.  64 problems of 16 to 1024 in BF16 (64 MB): 35 us, 38
-// without these, 37.3 with loads where they are used.
+// for it are taken once, rows and columns past the operand are only zeroed and
+// two squarings go in an instruction.  64 problems of 16 to 1024 in BF16 (64 MB):
+// 36.3 us, 38.5 without these.  (Loading the next k-block ahead: 35 us there, but
+// 64 instead of 48 registers leave four CTAs per SM instead of five, and 1024
+// problems take 788 us instead of 772; five CTAs with spills 810.)
 constexpr int STRIP_ROWS = 32;
 
 // A rows 128 rb + 32 s .. + 31 of problem P.  Warp w owns rows 4w .. 4w + 3
@@ -856,10 +857,9 @@ __device__ __forceinline__ bool a_strip(const Common& cm, const Level& lv, const
       }
     }
   };
-  float t[4][BK / 32], next[4][BK / 32];  // the next k-block's loads are in flight
-  load(0, t);
+  float t[4][BK / 32];
   for (int kb = 0; kb < P.KB; ++kb, dst += IMG_BYTES) {
-    load(min(kb + 1, P.KB - 1), next);
+    load(kb, t);
     __syncwarp();  // the previous k-block's reads of wsm are done
 #pragma unroll
     for (int r = 0; r < 4; ++r)
@@ -884,10 +884,6 @@ __device__ __forceinline__ bool a_strip(const Common& cm, const Level& lv, const
     PK::pack(v[0], hi, lo);
     *reinterpret_cast<uint4*>(dst) = hi;
     if constexpr (MODE == MODE_3XTF32) *reinterpret_cast<uint4*>(dst + P.a_plane) = lo;
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int h = 0; h < BK / 32; ++h) t[r][h] = next[r][h];
   }
   return bad;
 }
@@ -972,11 +968,10 @@ __device__ __forceinline__ bool b_strip(const Common& cm, const Level& lv, const
       }
     }
   };
-  float t[BK / 8], next[BK / 8];  // the next k-block's loads are in flight
-  load(0, t);
+  float t[BK / 8];
   for (int kb = 0; kb < P.KB; ++kb, dst += IMG_BYTES) {
     float* st = sm + (kb & 1) * (BK * TS);
-    load(min(kb + 1, P.KB - 1), next);
+    load(kb, t);
     if (inv_ok) {
 #pragma unroll
       for (int i = 0; i < BK / 8; ++i)
@@ -996,8 +991,6 @@ __device__ __forceinline__ bool b_strip(const Common& cm, const Level& lv, const
     PK::pack(v[0], hi, lo);
     *reinterpret_cast<uint4*>(dst) = hi;
     if constexpr (MODE == MODE_3XTF32) *reinterpret_cast<uint4*>(dst + P.b_plane) = lo;
-#pragma unroll
-    for (int i = 0; i < BK / 8; ++i) t[i] = next[i];
   }
   return bad;
 }
