@@ -161,8 +161,7 @@ def make_opts(p_log2=tuple(range(7)), compute="bf16", tau=None, scaling=2, diag_
     if not 1 <= len(pl) <= PN_MAX_P:
         raise ValueError("p family must have 1..16 entries")
     o.n_p = len(pl)
-    for q, v in enumerate(pl):
-        o.p_log2[q] = v
+    o.p_log2[:len(pl)] = pl
     o.tau = 0.0 if tau is None else float(tau)
     o.compute = COMPUTE_NAMES[compute] if isinstance(compute, str) else int(compute)
     o.scaling = int(scaling)
