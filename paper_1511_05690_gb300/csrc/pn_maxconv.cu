@@ -63,49 +63,6 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, __dmul_rn(a.y, b.y)), fma(a.x, b.y, -__dmul_rn(a.y, b.x)));
 }
 
-// In-place radix-2 decimation-in-time FFT of a[0..L) (L = 2^logL) held in
-// bit-reversed order; natural order on return; unscaled.  INV selects the
-// inverse (conjugate twiddles).  tw[k * tws] = exp(-2 pi i k / L).  The first
-// two stages (twiddles 1 and -+i) run as one multiply-free radix-4 pass.
-template <bool INV>
-__device__ void fft_dit(double2* a, const double2* tw, int logL, int tws) {
-  const int L = 1 << logL;
-  int s0 = 0;
-  if (logL >= 2) {
-    for (int g = threadIdx.x; g < (L >> 2); g += static_cast<int>(blockDim.x)) {
-      double2* q = a + 4 * g;
-      const double2 a0 = q[0], a1 = q[1], a2 = q[2], a3 = q[3];
-      const double2 b0 = make_double2(a0.x + a1.x, a0.y + a1.y);
-      const double2 b1 = make_double2(a0.x - a1.x, a0.y - a1.y);
-      const double2 b2 = make_double2(a2.x + a3.x, a2.y + a3.y);
-      const double2 b3 = make_double2(a2.x - a3.x, a2.y - a3.y);
-      // forward: t = -i b3; inverse: t = +i b3
-      const double2 t = INV ? make_double2(-b3.y, b3.x) : make_double2(b3.y, -b3.x);
-      q[0] = make_double2(b0.x + b2.x, b0.y + b2.y);
-      q[2] = make_double2(b0.x - b2.x, b0.y - b2.y);
-      q[1] = make_double2(b1.x + t.x, b1.y + t.y);
-      q[3] = make_double2(b1.x - t.x, b1.y - t.y);
-    }
-    __syncthreads();
-    s0 = 2;
-  }
-  for (int s = s0; s < logL; ++s) {
-    const int h = 1 << s;                     // half span
-    const int step = ((L >> 1) >> s) * tws;   // twiddle stride: L / (2h)
-    for (int b = threadIdx.x; b < (L >> 1); b += static_cast<int>(blockDim.x)) {
-      const int j = b & (h - 1);
-      const int i0 = ((b >> s) << (s + 1)) + j;
-      const int i1 = i0 + h;
-      const double2 w = tw[j * step];
-      const double2 t = INV ? cmulc(w, a[i1]) : cmul(w, a[i1]);
-      const double2 u = a[i0];
-      a[i0] = make_double2(u.x + t.x, u.y + t.y);
-      a[i1] = make_double2(u.x - t.x, u.y - t.y);
-    }
-    __syncthreads();
-  }
-}
-
 // (S)^(1/2^plog): plog correctly rounded FP32 square roots of float(S) for
 // S >= 1e-30 (the output is FP32; relative error about (plog + 1) 2^-24),
 // FP64 square roots below that (only unstable indices at the smallest p).
@@ -172,30 +129,13 @@ __device__ void direct_levels(const MaxconvArgs& ma, const float* x, const float
   res[m] = static_cast<uint8_t>(ma.p_log2[qs] | (stable ? 0 : 0x80));
 }
 
-// Z_k from A_k and A_(N-k) (the spectra of the packed real pair).
-__device__ __forceinline__ double2 spec_z(double2 ak, double2 an) {
-  const double2 X = make_double2(0.5 * (ak.x + an.x), 0.5 * (ak.y - an.y));
-  const double2 Y = make_double2(0.5 * (ak.y + an.y), -0.5 * (ak.x - an.x));
-  return cmul(X, Y);
-}
-
-// 4 spec_z(a, b), the halves left out (powers of two, exact).
+// 4 Z_k = 4 X_k Y_k from a = A_k and b = A_(N-k), the spectra of the packed real
+// pair: X = (a + conj b) / 2, Y = (a - conj b) / (2i); the halves are left out
+// (powers of two, exact).
 __device__ __forceinline__ double2 spec_z4(double2 a, double2 b) {
   const double2 s = make_double2(a.x + b.x, a.y - b.y);
   const double dy = a.y + b.y, ndx = b.x - a.x;  // -i (a - conj b) = (dy, ndx)
   return make_double2(fma(s.x, dy, -__dmul_rn(s.y, ndx)), fma(s.x, ndx, __dmul_rn(s.y, dy)));
-}
-
-// V_k = (Z_k + conj Z_(M-k)) / 2 + i conj(W^k) (Z_k - conj Z_(M-k)) / 2, w = W^k.
-__device__ __forceinline__ double2 spec_v(double2 zk, double2 zmk, double2 w) {
-  const double2 e = make_double2(0.5 * (zk.x + zmk.x), 0.5 * (zk.y - zmk.y));
-  const double2 d = make_double2(0.5 * (zk.x - zmk.x), 0.5 * (zk.y + zmk.y));
-  const double2 o = cmulc(w, d);  // O_k = conj(W^k) d
-  return make_double2(e.x - o.y, e.y + o.x);
-}
-
-__device__ __forceinline__ int bitrev(int k, int logN) {
-  return logN == 0 ? 0 : static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - logN));
 }
 
 __device__ __forceinline__ float pow_f32(float v, int plog) {
@@ -204,8 +144,8 @@ __device__ __forceinline__ float pow_f32(float v, int plog) {
 }
 
 // One level of the FFT convolution in shared memory: a = x'^p + i y'^p (zero
-// padded; powers in FP32), forward FFT of length N, the spectrum of the ring convolution, inverse at half length.  On return
-// S_m = (m odd ? a[m/2].y : a[m/2].x) * 2 / N.
+// padded; powers in FP32), forward FFT of length N, the spectrum of the ring
+// convolution, inverse at half length.
 //
 // The spectrum: X_k = (A_k + conj A_(N-k)) / 2, Y_k = (A_k - conj A_(N-k)) /
 // (2i), Z = X Y (Hermitian: the convolution is real).  Its inverse runs at
@@ -215,47 +155,11 @@ __device__ __forceinline__ float pow_f32(float v, int plog) {
 // V_k = E_k + i O_k = (Z_k + conj Z_(M-k)) / 2 + i W^-k (Z_k - conj Z_(M-k)) / 2
 // is the DFT of v_j = S_2j + i S_(2j+1).  Thread work: k and M - k together
 // (reads A at k, N - k, M - k, M + k).
-__device__ void conv_level(double2* a, const double2* tw, const MaxconvArgs& ma, const float* x,
-                           const float* y, float isx, float isy, int plog) {
-  const int N = 1 << ma.logN;
-  const int tid = threadIdx.x, nt = static_cast<int>(blockDim.x);
-  for (int k = tid; k < N; k += nt) {
-    float xr = 0.0f, yr = 0.0f;
-    if (k < ma.nx) xr = pow_f32(x[k] * isx, plog);
-    if (k < ma.ny) yr = pow_f32(y[k] * isy, plog);
-    a[bitrev(k, ma.logN)] = make_double2(static_cast<double>(xr), static_cast<double>(yr));
-  }
-  __syncthreads();
-  fft_dit<false>(a, tw, ma.logN, 1);
-  const int M = N >> 1;
-  constexpr int QUADS = FFT_NMAX / 4 / FFT_THREADS + 1;
-  double2 vk[QUADS], vm[QUADS];
-  for (int u = 0; u < QUADS; ++u) {
-    const int k = tid + u * nt;
-    if (k <= (M >> 1)) {
-      const double2 zk = spec_z(a[k], a[(N - k) & (N - 1)]);
-      const double2 zm = spec_z(a[M - k], a[M + k]);
-      vk[u] = spec_v(zk, zm, tw[k]);
-      vm[u] = spec_v(zm, zk, (M - k) < M ? tw[M - k] : make_double2(1.0, 0.0));
-    }
-  }
-  __syncthreads();
-  for (int u = 0; u < QUADS; ++u) {
-    const int k = tid + u * nt;
-    if (k <= (M >> 1)) {
-      a[bitrev(k, ma.logN - 1)] = vk[u];
-      if (k != 0 && (M - k) != k) a[bitrev(M - k, ma.logN - 1)] = vm[u];
-    }
-  }
-  __syncthreads();
-  fft_dit<true>(a, tw, ma.logN - 1, 2);
-}
-
-// ---- transforms in registers.  The same radix-2 butterflies, twiddles and
-// operation order as fft_dit / conv_level (in FP64 every value has the same
-// bits), but eight values per thread stay in registers for three stages, so a
-// transform of 2^13 makes 9 passes over shared memory with a barrier each
-// instead of 28, and nothing is permuted: the forward transform reads natural
+//
+// Radix-2 butterflies, decimation in time, eight values per thread in registers
+// for three stages, so that a level of N = 2^13 makes 9 passes over shared memory
+// with a barrier each instead of 28 (one per stage), and nothing is permuted: the
+// forward transform reads natural
 // order and leaves frequency k at address bitrev(k); the last forward stage
 // pairs the addresses of k and k + N/2, which the spectrum needs together
 // with those of N - k and N/2 - k, so it is fused into the spectrum; the
@@ -421,7 +325,7 @@ __device__ __forceinline__ void first_stages8(double2 (&v)[8], double2 w1, doubl
 
 // R stages s .. s + R - 1 of a transform of 2^lg values on the 2^R values
 // v[r] of one group; v[r] sits at position j + (r << s) within its block of
-// 2^(s + R) (positions as in fft_dit).  tw[k << tsh] = exp(-2 pi i k / 2^lg).
+// 2^(s + R) (position: the bit-reversed sample index).  tw[k << tsh] = exp(-2 pi i k / 2^lg).
 template <int R, bool INV, typename C>
 __device__ __forceinline__ void group_stages(C (&v)[1 << R], const C* tw, int lg, int tsh, int s,
                                              int j) {
@@ -477,7 +381,19 @@ __device__ __forceinline__ void inv_pass(C* a, const C* tw, int lg, int s) {
   __syncthreads();
 }
 
-// Inverse stages 0 to 2 (first_stages8), FP64.
+// Stages 0 to 2 (first_stages8), FP64: forward; inverse on the even addresses.
+__device__ __forceinline__ void fwd_first_pass(double2* a, const double2* tw, int lg) {
+  const int ng = 1 << (lg - 3);
+  for (int g = threadIdx.x; g < ng; g += blockDim.x) {
+    double2 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = a[slot(g + rev_bits(r, 3) * ng)];
+    first_stages8<false, false>(v, tw[ng], tw[3 * ng]);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) a[slot(g + rev_bits(r, 3) * ng)] = v[r];
+  }
+  __syncthreads();
+}
 __device__ __forceinline__ void inv_first_pass(double2* a, const double2* tw, int lg) {
   const double2 w1 = tw[2 << (lg - 3)], w3 = tw[6 << (lg - 3)];
   for (int g = threadIdx.x; g < (1 << (lg - 3)); g += blockDim.x) {
@@ -492,8 +408,8 @@ __device__ __forceinline__ void inv_first_pass(double2* a, const double2* tw, in
 }
 
 // The spectrum from the packed pair's transform (all but its last stage done)
-// to the half-length sequence 8 V_k in the even addresses; see conv_level.
-// The halves of the formulas there are left out: a power of two, exact.
+// to the half-length sequence 8 V_k in the even addresses (formulas above).
+// Their halves are left out: a power of two, exact.
 template <typename C>
 __device__ __forceinline__ void spectrum_pass(C* a, const C* tw, int lg) {
   const int lm = lg - 1, M = 1 << lm;
@@ -540,6 +456,10 @@ __device__ __forceinline__ void spectrum_pass(C* a, const C* tw, int lg) {
 // pass's loop outgrows the instruction cache (a third of the fetches missed)
 // and its registers allow half the warps.
 __device__ __forceinline__ void conv_passes(double2* a, const double2* tw, int lg, int s) {
+  if (s == 0 && lg >= 4) {
+    fwd_first_pass(a, tw, lg);
+    s = 3;
+  }
   for (; s + 3 <= lg - 1; s += 3) fwd_pass<3>(a, tw, lg, s);
   if (s + 2 == lg - 1) fwd_pass<2>(a, tw, lg, s);
   else if (s + 1 == lg - 1) fwd_pass<1>(a, tw, lg, s);
@@ -616,12 +536,16 @@ __device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw,
   __shared__ unsigned long long open_terms;
   __shared__ int n_open;
   const int N = 1 << ma.logN, tid = threadIdx.x, nt = static_cast<int>(blockDim.x);
-  const double invM = 2.0 / N;
+  const double scale = 0.25 / N;  // 2 / N, and the spectrum's 8
   __syncthreads();
   for (int k = tid; k < (N >> 1); k += nt) tw[k] = g_twiddle[k << (FFT_LOG_NMAX - ma.logN)];
   for (; q >= 0; --q) {
     const int plog = ma.p_log2[q];
-    conv_level(a, tw, ma, x, y, isx, isy, plog);
+    for (int k = tid; k < N; k += nt)
+      a[slot(k)] = make_double2(k < ma.nx ? pow_f32(x[k] * isx, plog) : 0.0f,
+                                k < ma.ny ? pow_f32(y[k] * isy, plog) : 0.0f);
+    __syncthreads();
+    conv_passes(a, tw, ma.logN, 0);
     // selection: first (largest) p with S >= tau; the smallest p takes the rest
     if (tid == 0) {
       open_terms = 0ull;
@@ -631,7 +555,8 @@ __device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw,
     unsigned long long my_terms = 0ull;
     for (int m = tid; m < ma.nz; m += nt) {
       if (res[m] != 0xFF) continue;
-      const double S = ((m & 1) ? a[m >> 1].y : a[m >> 1].x) * invM;
+      const double2 v = a[slot(m & ~1)];
+      const double S = ((m & 1) ? v.y : v.x) * scale;
       const bool stable = S >= ma.tau;
       if (stable || q == 0) {
         z[m] = static_cast<float>(sxy * root_pow2(S, plog));
@@ -673,8 +598,8 @@ __device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw,
 // FP64 transforms give.
 // Per problem of n = 4096 (one CTA, P = {1..64}): 62 us, of which the transforms
 // take 37 (issue slots: about 50 instructions per butterfly), against 240 by
-// FP64 transforms at 78 % of the FP64 pipe; 1024 problems 0.60 ms (0.43 where no
-// problem falls back to FP64), by FP64 transforms 1.66.
+// FP64 transforms at 78 % of the FP64 pipe; 1024 problems 0.54 to 0.61 ms (0.42
+// where no problem falls back to FP64), all by FP64 transforms 1.55.
 constexpr int MC_THREADS = 1024;
 constexpr int FF_SMALL_MAX = 512;  // indices summed directly, at most
 __global__ void __launch_bounds__(MC_THREADS, 1)
