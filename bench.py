@@ -78,9 +78,9 @@ P_LOG2 = list(range(7))
 def launches_per_step(args):
     """maxima + (images, GEMM) per level; the r = 2 projection adds
     a level at 3p/4 below every p whose p/2 and p/4 are in P; the affine
-    correction its two fit kernels."""
+    correction its three fit kernels."""
     levels = len(P_LOG2) + (len(P_LOG2) - 2 if args.estimator == 2 else 0)
-    return 1 + 2 * levels + (2 if args.correction == 2 else 0)
+    return 1 + 2 * levels + (3 if args.correction == 2 else 0)
 
 
 def workload_name(n, compute, estimator=0, correction=0, n_fit=0):

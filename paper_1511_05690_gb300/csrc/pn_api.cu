@@ -426,6 +426,9 @@ pn_status run_pnorm(int64_t M, int64_t N, int64_t K, const float* A, int64_t lda
       fa.scls = reinterpret_cast<int32_t*>(ws + L.off_scls);
       fa.coef = reinterpret_cast<float*>(ws + L.off_coef);
       fa.user_coef = o->fit_coef;
+      // partial sums in the state array, which the GEMM below is the first to write
+      fa.part = reinterpret_cast<float*>(ws + L.off_state);
+      fa.part_floats = M * (int64_t)L.state_ld;
       if ((e = launch_fit(cm, fa, stream))) return PN_ECUDA;
     }
     if (lv.is_top && o->ev_gemm_begin)

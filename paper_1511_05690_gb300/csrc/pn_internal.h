@@ -107,6 +107,8 @@ struct FitArgs {
   int32_t* scls;      // [n_fit]: each sample's p* class (-1: entry outside the product)
   float* coef;        // [PN_MAX_P][2]
   float* user_coef;   // optional copy for the caller
+  float* part;        // partial sums of k_fit_stream: [range][n_p + 1][n_fit]
+  int64_t part_floats;  // room there
 };
 
 // Control of one p level (one p of the family).
