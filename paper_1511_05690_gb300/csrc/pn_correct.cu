@@ -342,12 +342,15 @@ __global__ void k_fit_solve(const __grid_constant__ FitArgs fa) {
 // its ring.  It needs whole aligned rows of B, a thread per sample and room for
 // the partial sums, and reads all of B where k_fit_samples reads a sector per
 // term: B's rows at the copy rate cost less up to about 26 columns per sample
-// (measured at 8 columns per sample; the line is drawn at 16).
+// (1024 samples, in us, stream with merge against a block per sample: n = 16384
+// 246 / 285, 8192 91 / 136, 4096 63 / 70); below 4 M terms the merge costs more than the
+// scattered reads.
 constexpr int STREAM_SMEM = 220 * 1024;
 static int fit_ranges(const Common& cm, const FitArgs& fa, int* stages) {
   const Prob& P = cm.single;
   constexpr int a_bytes = ((STREAM_K * STREAM_LD + 31) & ~31) * 4;
-  if (fa.n_fit < 128 || fa.n_fit > STREAM_THREADS || P.K < 1024 || P.N > 16 * fa.n_fit) return 0;
+  if (fa.n_fit > STREAM_THREADS || (int64_t)fa.n_fit * P.K < (4 << 20) || P.N > 16 * fa.n_fit)
+    return 0;
   if ((P.N & 3) || (P.ldb & 3) || (reinterpret_cast<uintptr_t>(P.B) & 15)) return 0;
   const int n = (STREAM_SMEM - a_bytes) / (P.N * 4);
   if (n < 2) return 0;

@@ -11,8 +11,8 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("M,N,K,n_fit", [(300, 512, 1024, 128), (257, 260, 1500, 1024),
-                                         (1024, 2048, 2000, 1000), (2048, 4096, 4097, 700)])
+@pytest.mark.parametrize("M,N,K,n_fit", [(300, 512, 16400, 260), (257, 260, 4100, 1024),
+                                         (1024, 2048, 4200, 1000), (2048, 4096, 6001, 700)])
 @pytest.mark.parametrize("compute", ["bf16", "e4m3"])
 def test_stream_equals_block_per_sample(M, N, K, n_fit, compute):
     if not torch.cuda.is_available():
