@@ -565,8 +565,12 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
         });
     const int buf = s & (ACC_BUFS - 1);
     if (t == 0) mma_commit(&cx.acc_full[buf]);
-    if (warp >= 2 && warp < 2 + 4 * NG)
+    if (warp >= 2 && warp < 2 + 4 * NG) {
       run_epilogue<MODE, BN, 0, 1, NG, false, true>(cm, lv, cx, 1, false, s, Ready{nullptr, 0, 0});
+      // the staging buffers were written by ordinary stores, and the next
+      // level's tensor copies (async proxy) write the same bytes of the raw ring
+      fence_proxy_async_smem();
+    }
     __syncthreads();
     if (*cx.abort_flag || !*s_left) break;  // uniform: nothing writes either before the next barrier
     __syncthreads();
