@@ -87,7 +87,7 @@ struct Common {
   uint64_t timeout_ns;
   int32_t debug_flags;
   int32_t n_levels;
-  int32_t fp64_near;  // FP64 selection/root for entries with S < 10 tau (FP32-range formats)
+  int32_t fp64_near;  // roots to FP64 accuracy for entries with S < 10 tau (FP32-range formats)
   int32_t grad_axis;  // gradient epilogue: 0 = scale per output row (r), 1 = per column (c)
   int32_t post;       // APSP squaring: 1 = C_ii = 1, 2 = also C = min(C, 1)
   int32_t corr;       // bias correction: 0 none, 1 divide by K^(1/p*), 2 affine per p* class
