@@ -42,3 +42,24 @@ def test_near_tau(pn, compute, q, shape):
                                tau=4.0)
     C, S = C.cpu().numpy(), S.cpu().numpy()
     assert np.array_equal(C, _fp64_roots(S, q))
+
+
+@pytest.mark.parametrize("q", [1, 2, 3, 6, 7, 9])
+@pytest.mark.parametrize("compute", ["f32", "tf32", "bf16"])
+def test_large_sums(pn, compute, q):
+    # unscaled operands whose sums reach from 2^100 to 2^128 and past it
+    p = 2.0 ** q
+    g = torch.Generator().manual_seed(q)
+    a = torch.exp2((50 + 14.2 * torch.rand((200, 1), generator=g)) / p)
+    b = torch.exp2((50 + 14.2 * torch.rand((1, 300), generator=g)) / p)
+    C, _, S = pn.maxprod_pnorm(a.cuda(), b.cuda(), p_log2=(q,), compute=compute, scaling=0)
+    C, S = C.cpu().numpy(), S.cpu().numpy()
+    want = S.astype(np.float64) ** (1.0 / p)
+    assert np.array_equal(np.isinf(C), np.isinf(S)) and np.isinf(S).any()
+    fin = np.isfinite(S)
+    # as test_gpu_root.py: half an ulp and one rounding; two hardware approximations
+    tol = 2.0 ** -23 if compute == "f32" else 2.0 ** -21 + 2.0 ** -15 / p
+    assert np.all(np.abs(C[fin] - want[fin]) <= tol * want[fin])
+    if compute == "f32":
+        big = fin & (S >= 2.0 ** 120)
+        assert big.any() and np.array_equal(C[big], _fp64_roots(S[big], q))
