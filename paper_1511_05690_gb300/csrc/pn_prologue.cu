@@ -16,6 +16,7 @@
 #include <cuda_fp8.h>
 
 #include "pn_image.cuh"
+#include "pn_split.h"
 
 namespace pn {
 
@@ -634,6 +635,9 @@ int sm_count() {
   return sms;
 }
 
+// CTAs of a launch that builds `total` tiles by tensor copies.
+int tma_ctas(int total) { return std::min(total, TMA_CTAS_32K * sm_count()); }
+
 template <int MODE>
 int launch_tma_t(const Common& cm, const Level& lv, void* stream, const OperandMaps& maps, int xa,
                  int xb) {
@@ -647,20 +651,24 @@ int launch_tma_t(const Common& cm, const Level& lv, void* stream, const OperandM
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
+  static_assert(CA::CTAS == TMA_CTAS_32K && CB::CTAS == TMA_CTAS_32K, "see tma_together");
   // the resident CTAs, shared out by the operands' tiles
-  const int total = xa + xb;
-  const int grid = total < CB::CTAS * sm_count() ? total : CB::CTAS * sm_count();
-  int n_a = xb == 0 ? grid : static_cast<int>(static_cast<int64_t>(grid) * xa / total);
-  if (xa > 0 && n_a == 0) n_a = 1;
-  if (xb > 0 && n_a == grid) n_a = grid - 1;
+  const int grid = tma_ctas(xa + xb);
+  const int n_a = xb == 0 ? grid : xa == 0 ? 0 : image_split(xa, xb, grid);
   const cudaError_t e = launch_pdl(k_image_tma<MODE>, dim3(grid), dim3(CB::THREADS), smem, stream, cm,
                                    lv, *reinterpret_cast<const CUtensorMap*>(&maps.a),
                                    *reinterpret_cast<const CUtensorMap*>(&maps.b), n_a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// The tensor-copy kernel takes at most TMA_MAX_OWNED tiles per SM.
+// The tensor-copy kernel takes at most TMA_MAX_OWNED tiles per SM, so that no CTA
+// owns more than TmaCfg::MAX_OWNED: one operand, both in one launch.
 bool tma_fits(int total) { return total <= TMA_MAX_OWNED * sm_count(); }
+bool tma_together(int xa, int xb) {
+  if (xa < 1 || xb < 1) return false;
+  const int n = tma_ctas(xa + xb), n_a = image_split(xa, xb, n);
+  return std::max(tiles_owned(xa, n_a), tiles_owned(xb, n - n_a)) <= TMA_MAX_OWNED / TMA_CTAS_32K;
+}
 
 // xa / xb: tiles of A / B to build (0: not this operand).
 int launch_tma(const Common& cm, const Level& lv, void* stream, const OperandMaps& maps, int xa,
@@ -1105,8 +1113,7 @@ int launch_images(const Common& cm, const Level& lv, void* stream, const Operand
   const int xa = cm.total_xa, xb = cm.total_xb;
   const bool ta = maps && maps->has_a && tma_fits(xa), tb = maps && maps->has_b && tma_fits(xb);
   int e = 0;
-  if (ta && tb && tma_fits(xa + xb))
-    return xa + xb > 0 ? launch_tma(cm, lv, stream, *maps, xa, xb) : 0;
+  if (ta && tb && tma_together(xa, xb)) return launch_tma(cm, lv, stream, *maps, xa, xb);
   if (ta && xa > 0) e = launch_tma(cm, lv, stream, *maps, xa, 0);
   if (!e && tb && xb > 0) e = launch_tma(cm, lv, stream, *maps, 0, xb);
   const int pa = ta ? 0 : xa, pb = tb ? 0 : xb;

@@ -1,0 +1,63 @@
+"""How the CTAs of the merged image launch are shared out between A and B: a CTA's
+list of tiles holds 2048 entries, and the busiest CTA sets the time.  The host
+function is compiled by itself, no GPU needed."""
+import ctypes
+import os
+import random
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_1511_05690_gb300", "csrc")
+LIST = 2048  # tiles per CTA
+CTAS = 304   # two on each of 152 SMs
+
+
+@pytest.fixture(scope="module")
+def split(tmp_path_factory):
+    d = tmp_path_factory.mktemp("split")
+    (d / "s.cpp").write_text(
+        '#include "pn_split.h"\n'
+        'extern "C" int split(long long a, long long b, int n) { return pn::image_split(a, b, n); }\n')
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "s.cpp"),
+                    "-o", str(d / "s.so")], check=True)
+    f = ctypes.CDLL(str(d / "s.so")).split
+    f.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
+    return f
+
+
+def _worst(xa, xb, n, ctas):
+    return max(-(-xa // n), -(-xb // (ctas - n)))
+
+
+def test_no_split_is_better(split):
+    rng = random.Random(1)
+    for _ in range(3000):
+        ctas = rng.choice([2, 3, 8, CTAS, rng.randint(2, CTAS)])
+        xa, xb = (int(2 ** rng.uniform(0, 20)) for _ in range(2))
+        if xa + xb < ctas:
+            ctas = max(2, xa + xb)
+        n = split(xa, xb, ctas)
+        assert 1 <= n < ctas
+        assert _worst(xa, xb, n, ctas) == min(_worst(xa, xb, m, ctas) for m in range(1, ctas))
+
+
+def test_one_tile_each_when_there_are_fewer_tiles_than_ctas(split):
+    for xa, xb in ((1, 1), (1, 200), (200, 1), (100, 150)):
+        assert split(xa, xb, xa + xb) == xa
+
+
+@pytest.mark.parametrize("M,N,K,bk", [
+    (1024, 160000, 20480, 64), (128, 19456, 131200, 64), (128, 20480, 16384, 64),
+    (19456, 128, 65600, 32), (128, 128 * 2400, 16384, 64)])
+def test_skewed_products(split, M, N, K, bk):
+    # by the rounded-down share one CTA took all of A: up to 4000 tiles and
+    # twice the others' part
+    kb = -(-K // bk)
+    xa, xb = -(-M // 128) * kb, -(-N // 128) * kb
+    n = split(xa, xb, CTAS)
+    worst, mean = _worst(xa, xb, n, CTAS), (xa + xb) / CTAS
+    assert worst == min(_worst(xa, xb, m, CTAS) for m in range(1, CTAS))
+    if mean <= LIST * 0.95:
+        assert worst <= LIST and worst <= 1.02 * mean + 1
