@@ -112,7 +112,8 @@ typedef struct pn_opts {
    * persistent launch (same results; for comparing the two).  Bit 3: the
    * persistent grouped launch also builds the top level's operand images
    * itself instead of taking them from the image kernels launched before it
-   * (same results). */
+   * (same results).  Bit 4: the one-launch small product never copies its first
+   * operand block (16-byte aligned rows; as bit 0). */
   int32_t debug_flags;
   /* Estimate of max_k u_k from the p-sums (Sec. 2.1):
    *   0 (default) = plain, (S^(p*))^(1/p*), an overestimate by at most

@@ -356,7 +356,7 @@ Level make_level(const Layout& L, const pn_opts* o, uint8_t* ws, const Schedule&
 constexpr int64_t FUSED_NS = 55000;
 int fused_bn(const pn_opts* o, int64_t M, int64_t N, int64_t K, bool aligned, int sms) {
   if (o->tile_m || o->tile_n || o->scaling == 1 || o->correction == 2 || o->estimator == 2 ||
-      o->debug_flags || host_tuned_bn(o->compute, M, N, K))
+      (o->debug_flags & ~16) || host_tuned_bn(o->compute, M, N, K))
     return 0;
   const int64_t rows = ceil_div(M, TILE_M);
   const int bn = rows * ceil_div(N, 64) <= sms ? 64 : rows * ceil_div(N, 128) <= sms ? 128 : 0;

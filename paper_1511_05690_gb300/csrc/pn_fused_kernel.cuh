@@ -193,11 +193,13 @@ struct RawRing {
 // Walks the raw blocks 0 .. count - 1 of tile (tm, tn): body(i, addr) with all
 // of block i in shared memory at addr, RAW - 1 blocks ahead in flight; done(i)
 // once every thread has finished the body of block i (and fenced its
-// shared-memory writes for the async proxy).  Called by every thread.
+// shared-memory writes for the async proxy).  Called by every thread.  drop_first
+// (test hook): block 0 is never copied.
 template <int BN, int RAW, typename Body, typename Done>
 __device__ __forceinline__ void raw_walk(const RawSrc& rs, RawRing& rr, const OperandMaps& maps,
-                                         const Ctx& cx, int32_t* status, int tm, int tn, int count,
-                                         int t, const Body& body, const Done& done) {
+                                         const Ctx& cx, int32_t* status, bool drop_first, int tm,
+                                         int tn, int count, int t, const Body& body,
+                                         const Done& done) {
   RawWalk<BN> w;
   if (!rr.tma) w.init(rs, t);
   int put = rr.slot;
@@ -209,6 +211,10 @@ __device__ __forceinline__ void raw_walk(const RawSrc& rs, RawRing& rr, const Op
       } else if (!mbar_wait(&rr.full[rr.slot], rr.phase, cx.tmo, cx.abort_flag)) {
         *cx.abort_flag = 1;
         set_status(status, PN_ETIMEOUT);
+        // the walk goes on to its end: thread 0 still waits for every block, so
+        // that no copy outlives the CTA's memory
+        if (t == 0 && !mbar_wait_drain(&rr.full[rr.slot], rr.phase, cx.tmo) && drop_first)
+          mbar_arrive(&rr.full[rr.slot]);  // in place of the block that was left out
       }
       __syncthreads();  // block i has landed, block i - 1 is finished, for every thread
       if (i > 0) done(i - 1);
@@ -218,7 +224,7 @@ __device__ __forceinline__ void raw_walk(const RawSrc& rs, RawRing& rr, const Op
     if (n < count) {
       if (!rr.tma) {
         w.issue(rs, dst, n, t);
-      } else if (t == 0) {
+      } else if (t == 0 && !(drop_first && n == 0)) {
         mbar_arrive_expect_tx(&rr.full[put], raw_bytes(BN));
         tma_load_2d(dst, &maps.a, n * RAW_K, tm * TILE_M, &rr.full[put]);
         tma_load_2d(dst + TILE_M * 128, &maps.b, tn * BN, n * RAW_K, &rr.full[put]);
@@ -381,6 +387,7 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
   rr.slot = 0;
   rr.phase = 0;
   rr.tma = maps.has_a && maps.has_b;
+  const bool drop_first = (cm.debug_flags & 16) != 0;
   int32_t* const s_left = reinterpret_cast<int32_t*>(ctrl + 320);
   float* const s_scale = reinterpret_cast<float*>(ctrl + 512);  // maxima as bits first
   cx.rs = s_scale;
@@ -420,7 +427,7 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
     for (int j = 0; j < 2; ++j) oa[j] = ra * 128 + ((((t & 3) * 2 + j) ^ (ra & 7)) << 4);
     const uint32_t ob = TILE_M * 128 + ((t / BN) * KB_T * BN + n) * 4;
     raw_walk<BN, RAW>(
-        rs, rr, maps, cx, cm.status, tm, tn, (P.K + RAW_K - 1) / RAW_K, t,
+        rs, rr, maps, cx, cm.status, drop_first, tm, tn, (P.K + RAW_K - 1) / RAW_K, t,
         [&](int, uint32_t blk) {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -432,9 +439,10 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
             ub = max(ub, __float_as_uint(lds_f32(blk + ob + e * BN * 4)));
         },
         [](int) {});
-    if (ua > DOMAIN_MAX_BITS)  // over the whole row (it exists: others are zeros)
+    // over the whole row or column (others are zeros, but after a copy that never landed)
+    if (ua > DOMAIN_MAX_BITS && ra < rs.rows)
       ua = take_exact(exact_max_bits(rs.a + ra * rs.lda, 1, P.K), bad);
-    if (ub > DOMAIN_MAX_BITS) ub = take_exact(exact_max_bits(rs.b + n, rs.ldb, P.K), bad);
+    if (ub > DOMAIN_MAX_BITS && n < rs.cols) ub = take_exact(exact_max_bits(rs.b + n, rs.ldb, P.K), bad);
     ua = max(ua, __shfl_xor_sync(0xffffffffu, ua, 1));
     ua = max(ua, __shfl_xor_sync(0xffffffffu, ua, 2));
     if ((t & 3) == 0) smax[ra] = ua;
@@ -494,7 +502,7 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
     const uint32_t acc = cx.tmem_base + (s & (ACC_BUFS - 1)) * BN;
     int mma_stage = stage;  // the stage of the next block to multiply
     raw_walk<BN, RAW>(
-        rs, rr, maps, cx, cm.status, tm, tn, P.KB * SUBS, t,
+        rs, rr, maps, cx, cm.status, drop_first, tm, tn, P.KB * SUBS, t,
         [&](int i, uint32_t blk) {
           const int sub = SUBS == 1 ? 0 : i % SUBS;
           if (sub == 0 && !aborted &&
@@ -576,12 +584,9 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
     __syncthreads();
   }
   if (*cx.abort_flag && t == 0) {
-    // no MMA or copy may outlive the CTA's memory (a copy lands within
-    // microseconds; all are waited for where nothing timed out)
+    // no MMA may outlive the CTA's memory (raw_walk has waited for the copies)
     mma_commit(cx.drain);
     mbar_wait_drain(cx.drain, 0, cx.tmo);
-    const uint64_t t0 = globaltimer_ns();
-    while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
   }
   ctx_teardown<BN>(cx);
 }
