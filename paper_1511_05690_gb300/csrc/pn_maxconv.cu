@@ -88,20 +88,34 @@ __device__ __forceinline__ int terms_of(int m, int nx, int ny) {
   return hi - lo + 1;
 }
 
-// Index m still open after level q: its p-sums for levels q-1 .. 0 summed
-// directly, sum_i (x'_i y'_(m-i))^p in FP64, then the selection rule.
-__device__ void direct_levels(const MaxconvArgs& ma, const float* x, const float* y, double isx,
-                              double isy, double sxy, int m, int q, float* z, uint8_t* res) {
-  double S[PN_MAX_P];
+// v >= 0 in FP64; a normal value without the conversion, which takes an FP64 slot.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v);
+  if (b != 0u && b < 0x00800000u) return static_cast<double>(v);
+  return b == 0u ? 0.0 : __hiloint2double((b >> 3) + 0x38000000u, b << 29);
+}
+
+// Index m still open after level q <= Q: its p-sums for levels q-1 .. 0 summed
+// directly, sum_i (x'_i y'_(m-i))^p in FP64, then the selection rule, by G = 1 lane or
+// the G = 32 of a warp (the terms in turn).  iss = the scales' reciprocals multiplied
+// (exactly), so that a term takes two FP64 products and no conversion, of about 16
+// FP64 instructions, which bound it.  The Q sums are held in registers: 16 of them
+// spill in a kernel of 64 registers.
+template <int G, int Q>
+__device__ __forceinline__ void direct_levels_q(const MaxconvArgs& ma, const float* x,
+                                                const float* y, double iss, double sxy,
+                                                int m, int q, float* z, uint8_t* res) {
+  double S[Q];
 #pragma unroll
-  for (int t = 0; t < PN_MAX_P; ++t) S[t] = 0.0;
+  for (int t = 0; t < Q; ++t) S[t] = 0.0;
+  const int lane = threadIdx.x & (G - 1);
   const int lo = m - ma.ny + 1 > 0 ? m - ma.ny + 1 : 0;
   const int hi = m < ma.nx - 1 ? m : ma.nx - 1;
-  for (int i = lo; i <= hi; ++i) {
-    double t = (static_cast<double>(x[i]) * isx) * (static_cast<double>(y[m - i]) * isy);
+  for (int i = lo + lane; i <= hi; i += G) {
+    double t = (widen(x[i]) * widen(y[m - i])) * iss;  // = x'_i y'_(m-i): both products are exact
     int lg = 0;
 #pragma unroll
-    for (int u = 0; u < PN_MAX_P; ++u) {
+    for (int u = 0; u < Q; ++u) {
       if (u < q) {
         while (lg < ma.p_log2[u]) {
           t *= t;
@@ -114,19 +128,29 @@ __device__ void direct_levels(const MaxconvArgs& ma, const float* x, const float
   int qs = -1;
   double s_sel = 0.0;
 #pragma unroll
-  for (int u = PN_MAX_P - 1; u >= 0; --u) {
-    if (u < q && qs < 0 && S[u] >= ma.tau) {
-      qs = u;
-      s_sel = S[u];
+  for (int u = Q - 1; u >= 0; --u) {
+    if (u < q && qs < 0) {
+      if constexpr (G == 32) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) S[u] += __shfl_xor_sync(0xffffffffu, S[u], off);
+      }
+      if (u == 0 || S[u] >= ma.tau) {
+        qs = u;
+        s_sel = S[u];
+      }
     }
   }
-  const bool stable = qs >= 0;
-  if (!stable) {
-    qs = 0;
-    s_sel = S[0];
+  if (lane == 0) {
+    z[m] = static_cast<float>(sxy * root_pow2(s_sel, ma.p_log2[qs]));
+    res[m] = static_cast<uint8_t>(ma.p_log2[qs] | (s_sel >= ma.tau ? 0 : 0x80));
   }
-  z[m] = static_cast<float>(sxy * root_pow2(s_sel, ma.p_log2[qs]));
-  res[m] = static_cast<uint8_t>(ma.p_log2[qs] | (stable ? 0 : 0x80));
+}
+template <int G = 1>
+__device__ __forceinline__ void direct_levels(const MaxconvArgs& ma, const float* x,
+                                              const float* y, double iss, double sxy,
+                                              int m, int q, float* z, uint8_t* res) {
+  if (q <= 6) direct_levels_q<G, 6>(ma, x, y, iss, sxy, m, q, z, res);
+  else direct_levels_q<G, PN_MAX_P>(ma, x, y, iss, sxy, m, q, z, res);
 }
 
 // 4 Z_k = 4 X_k Y_k from a = A_k and b = A_(N-k), the spectra of the packed real
@@ -500,32 +524,21 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// direct_levels by a whole warp: lanes take the terms in turn (an index at the
-// edge has a few dozen at most, and one FP64 instruction of a warp takes 64
-// cycles however many lanes it has).
-__device__ void direct_levels_warp(const MaxconvArgs& ma, const float* x, const float* y,
-                                   double isx, double isy, double sxy, int m, int q, float* z,
-                                   uint8_t* res, int lane) {
-  const int lo = m - ma.ny + 1 > 0 ? m - ma.ny + 1 : 0;
-  const int hi = m < ma.nx - 1 ? m : ma.nx - 1;
-  // level by level from the largest p left: most indices stop at the first
-  for (int u = q - 1; u >= 0; --u) {
-    double S = 0.0;
-    for (int i = lo + lane; i <= hi; i += 32) {
-      double t = (static_cast<double>(x[i]) * isx) * (static_cast<double>(y[m - i]) * isy);
-      for (int s = 0; s < ma.p_log2[u]; ++s) t *= t;
-      S += t;
-    }
-    S = warp_sum(S);
-    const bool stable = S >= ma.tau;
-    if (stable || u == 0) {
-      if (lane == 0) {
-        z[m] = static_cast<float>(sxy * root_pow2(S, ma.p_log2[u]));
-        res[m] = static_cast<uint8_t>(ma.p_log2[u] | (stable ? 0 : 0x80));
-      }
-      return;
-    }
-  }
+// The `count` open indices of list after level q, block-wide: those of 64 terms or
+// more by a warp each, the others by a thread each (an FP64 instruction of a warp
+// takes the same time however many lanes have work, and a warp's sums meet at the
+// end).  1024 problems of 4096 values in [1/16, 1]: 2.8 ms, 6.6 with a thread for
+// every index, 5.0 when 512 threads of twice the registers ran them.
+__device__ void direct_open(const MaxconvArgs& ma, const float* x, const float* y, double iss,
+                            double sxy, const int* list, int count, int q, float* z,
+                            uint8_t* res) {
+  const int tid = threadIdx.x, nt = static_cast<int>(blockDim.x);
+  for (int e = tid >> 5; e < count; e += nt >> 5)
+    if (terms_of(list[e], ma.nx, ma.ny) >= 64)
+      direct_levels<32>(ma, x, y, iss, sxy, list[e], q, z, res);
+  for (int e = tid; e < count; e += nt)
+    if (terms_of(list[e], ma.nx, ma.ny) < 64)
+      direct_levels<1>(ma, x, y, iss, sxy, list[e], q, z, res);
 }
 
 // The levels q .. 0 of one problem by FP64 transforms, for the indices still
@@ -576,9 +589,7 @@ __device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw,
         if (res[m] == 0xFF) list[atomicAdd(&n_open, 1)] = m;
       __syncthreads();
       const int cnt = n_open;
-      for (int e = tid; e < cnt; e += nt)
-        direct_levels(ma, x, y, static_cast<double>(isx), static_cast<double>(isy), sxy, list[e],
-                      q, z, res);
+      direct_open(ma, x, y, static_cast<double>(isx) * isy, sxy, list, cnt, q, z, res);
       break;
     }
   }
@@ -614,6 +625,7 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
   __shared__ int n_small, n_open, redo;
   __shared__ int small[FF_SMALL_MAX];
   __shared__ double small_S[FF_SMALL_MAX];
+  __shared__ unsigned s_large[2];
   const int b = blockIdx.x;
   const float* x = ma.x + (int64_t)b * ma.ldx;
   const float* y = ma.y + (int64_t)b * ma.ldy;
@@ -649,6 +661,7 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
     red[1][warp] = my;
   }
   for (int m = tid; m < ma.nz; m += nt) res[m] = 0xFF;
+  if (tid < 2) s_large[tid] = 0u;
   __syncthreads();
   mx = my = 0.0f;
   for (int w = 0; w < nw; ++w) {
@@ -682,14 +695,36 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
   // thresholds beyond FP32: FP64 from the start
   bool ff = lg >= 5 && sxy_h >= 1e-30f && sxy_h <= 1e30f && tau >= 1e-30f && tau <= 1e6f;
   int q = ma.n_p - 1;
+  // A term of a sum that reaches theta (below, at least 2^-17 sqrt(log2 N / N), as the
+  // largest x'^p and y'^p are 1) has both its factors at or above least, so at
+  // most as many sums reach it as there are pairs of such factors.  Where the
+  // largest p leaves too few pairs, its transforms in two floats are not begun:
+  // they took 37 of the 232 us of a problem that falls back (1024 problems with
+  // one value in 100 not zero: 11.6 ms, 11.1 so).
+  const float least = 7.0e-6f * sqrtf(static_cast<float>(lg) / N) / min(ma.nx, ma.ny);
   for (; ff && q >= 0; --q) {
     const int plog = ma.p_log2[q];
+    unsigned large_x = 0, large_y = 0;
     for (int k = tid; k < N; k += nt) {
       const float xr = k < ma.nx ? pow_f32(x[k] * isx, plog) : 0.0f;
       const float yr = k < ma.ny ? pow_f32(y[k] * isy, plog) : 0.0f;
       a[slot(k)] = cff{f2_pack(xr, yr), 0ull};
+      large_x += xr >= least;
+      large_y += yr >= least;
+    }
+    if (q == ma.n_p - 1) {
+      large_x = __reduce_add_sync(0xffffffffu, large_x);
+      large_y = __reduce_add_sync(0xffffffffu, large_y);
+      if (lane == 0) {
+        atomicAdd(&s_large[0], large_x);
+        atomicAdd(&s_large[1], large_y);
+      }
     }
     __syncthreads();
+    if (q == ma.n_p - 1 && s_large[0] * s_large[1] + FF_SMALL_MAX < static_cast<unsigned>(ma.nz)) {
+      ff = false;
+      break;
+    }
     conv_passes(a, tw, lg);
     // the sums' root mean square
     constexpr int PER = FFT_NMAX / MC_THREADS;
@@ -785,9 +820,7 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
         if (res[m] == 0xFF) list[atomicAdd(&n_open, 1)] = m;
       __syncthreads();
       const int open = n_open;
-      for (int e = warp; e < open; e += nw)
-        direct_levels_warp(ma, x, y, static_cast<double>(isx), static_cast<double>(isy), sxy,
-                           list[e], q, z, res, lane);
+      direct_open(ma, x, y, static_cast<double>(isx) * isy, sxy, list, open, q, z, res);
       break;
     }
     __syncthreads();
@@ -1330,7 +1363,7 @@ __global__ void k_long_direct(const __grid_constant__ LongArgs la, int q) {
   const double isx = static_cast<double>(static_cast<float>(1.0 / sx));
   const double isy = static_cast<double>(static_cast<float>(1.0 / sy));
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < la.nz; m += gridDim.x * blockDim.x)
-    if (la.res[m] == 0xFF) direct_levels(ma, la.x, la.y, isx, isy, sx * sy, m, q, la.z, la.res);
+    if (la.res[m] == 0xFF) direct_levels(ma, la.x, la.y, isx * isy, sx * sy, m, q, la.z, la.res);
   if (blockIdx.x == 0 && threadIdx.x == 0) *la.done = q + 1;
 }
 
