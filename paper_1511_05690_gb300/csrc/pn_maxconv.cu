@@ -597,20 +597,25 @@ __device__ void maxconv_levels64(const MaxconvArgs& ma, double2* a, double2* tw,
 
 // One CTA per problem.  Per level the transforms run in two floats per value
 // (see above).  Their rounding adds noise to every S_m, independent of S_m's
-// own size: with R the root mean square of the S_m, its standard deviation is
-// at most sigma = 2^-45 sqrt(log2 N) R (measured 0.12 to 0.28 sigma, largest
-// value 1.2 sigma, N = 2^13), that of FP64 transforms sigma64 = 2^-53
-// sqrt(log2 N) R (measured 0.6).  An index with S_m >= theta = 2^28 sigma (16
-// sigma below 2^-24 of S_m) is rooted from it.  The others -- the outermost few,
-// which sum few terms -- get S_m by a direct FP64 sum, which has no such noise.
-// Where that sum lies within 3 sigma64 of tau (about one problem in 400), or
-// where too many indices lie below theta (wide ranges of values), the
-// problem's level and the rest run in FP64 transforms, so that p_sel is what
-// FP64 transforms give.
+// own size.  Its scale R: the products' and the inverse transform's rounding goes
+// with the root mean square of the S_m; x'^p and y'^p are transformed together, so
+// each spectrum has an error that goes with both their norms, which multiplied by
+// the spectra and transformed back comes to (|x'^p|^2 + |y'^p|^2) / sqrt(N) (more
+// than the first only where one vector outweighs the other); R^2 is the sum of
+// the squares.  The noise's standard deviation is at most sigma = 2^-45
+// sqrt(log2 N) R (measured 0.12 to 0.28 sigma, largest value 1.2 sigma, N = 2^13),
+// that of FP64 transforms sigma64 = 2^-53 sqrt(log2 N) R (measured 0.6).  An index
+// with S_m >= theta = 2^28 sigma (16 sigma below 2^-24 of S_m) is rooted from it.
+// The others -- the outermost few, which sum few terms -- get S_m by a direct
+// FP64 sum, which has no such noise.  Where that sum lies within 4 sigma64 of tau,
+// more than six of the noise's standard deviations (about one problem in 300), or
+// where too many indices lie below theta (wide ranges of values), the problem's
+// level and the rest run in FP64 transforms, so that p_sel is what FP64
+// transforms give.
 // Per problem of n = 4096 (one CTA, P = {1..64}): 62 us, of which the transforms
 // take 37 (issue slots: about 50 instructions per butterfly), against 240 by
-// FP64 transforms at 78 % of the FP64 pipe; 1024 problems 0.54 to 0.61 ms (0.42
-// where no problem falls back to FP64), all by FP64 transforms 1.55.
+// FP64 transforms at 78 % of the FP64 pipe; 1024 problems 0.55 to 0.62 ms (0.43
+// where no problem falls back to FP64), all by FP64 transforms 1.49.
 constexpr int MC_THREADS = 1024;
 constexpr int FF_SMALL_MAX = 512;  // indices summed directly, at most
 __global__ void __launch_bounds__(MC_THREADS, 1)
@@ -705,10 +710,12 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
   for (; ff && q >= 0; --q) {
     const int plog = ma.p_log2[q];
     unsigned large_x = 0, large_y = 0;
+    float sq = 0.0f;  // |x'^p|^2 + |y'^p|^2
     for (int k = tid; k < N; k += nt) {
       const float xr = k < ma.nx ? pow_f32(x[k] * isx, plog) : 0.0f;
       const float yr = k < ma.ny ? pow_f32(y[k] * isy, plog) : 0.0f;
       a[slot(k)] = cff{f2_pack(xr, yr), 0ull};
+      sq = fmaf(xr, xr, fmaf(yr, yr, sq));
       large_x += xr >= least;
       large_y += yr >= least;
     }
@@ -741,18 +748,27 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
       }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-    if (lane == 0) red[0][warp] = ss;
+    for (int off = 16; off > 0; off >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    }
+    if (lane == 0) {
+      red[0][warp] = ss;
+      red[1][warp] = sq;
+    }
     if (tid == 0) {
       s_terms = 0ull;
       n_small = n_open = redo = 0;
     }
     __syncthreads();
-    ss = 0.0f;
-    for (int w = 0; w < nw; ++w) ss += red[0][w];
-    const float noise = sqrtf(static_cast<float>(lg) * ss / N);
+    ss = sq = 0.0f;
+    for (int w = 0; w < nw; ++w) {
+      ss += red[0][w];
+      sq += red[1][w];
+    }
+    const float noise = sqrtf(static_cast<float>(lg) * fmaf(sq, sq, ss) / N);  // sqrt(log2 N) R
     const float theta = fmaxf(noise * 7.62939453e-6f, 4.0f * tau);           // 2^28 2^-45
-    const float near = noise * 3.33066907e-16f;  // 3 2^-53
+    const float near = noise * 4.44089210e-16f;  // 4 2^-53
     unsigned long long terms = 0ull;
 #pragma unroll
     for (int u = 0; u < PER; ++u) {

@@ -74,3 +74,22 @@ def test_against_direct_sums(kx, ky, nx, ny):
         hi = (S[q, at] + err[q, at]) ** r * scale
         tol = (q + 3) * 2.0 ** -24 * 1.5
         assert np.all((z[b] >= lo * (1 - tol) - 1e-44) & (z[b] <= hi * (1 + tol) + 1e-44))
+
+
+@pytest.mark.parametrize("nx,ny", [(8000, 150), (150, 8000), (4000, 60)])
+def test_one_vector_outweighs_the_other(nx, ny):
+    """A long vector of ones and small values against a single 1: the outputs are the
+    long vector's values, to one rounding (p = 1 leaves nothing of an error in S)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1511_05690_gb300 as pn
+    n, k = max(nx, ny), min(nx, ny)
+    g = torch.Generator().manual_seed(n)
+    v, one = torch.ones((40, n)), torch.zeros((40, k))
+    small = torch.exp2(-15 + torch.rand((40, n // 17), generator=g))
+    v[:, 5:5 + 16 * (n // 17):16] = small
+    one[:, 3] = 1.0
+    x, y = (v, one) if nx > ny else (one, v)
+    z, _ = pn.maxconv_pnorm(x.cuda(), y.cuda(), p_log2=(0,))
+    z = z.cpu()[:, 3:3 + n].double()
+    assert torch.all((z - v.double()).abs() <= 2.0 ** -24 * v)
