@@ -1951,23 +1951,38 @@ int maxconv_fft_smem_bytes(int logN) {
   return N * 16 + (N / 2) * 16 + N;  // data, twiddles, p_sel of up to N indices
 }
 
-// The device's table of FFT twiddle factors, filled on the first use.
-int ensure_twiddles(cudaStream_t s) {
+// The device's tables of FFT twiddle factors, filled on the first use: on a stream of
+// their own that is waited for, so that the tables are there for every stream and
+// thread once they are marked ready, and so that a first call under stream
+// capture fills them at once instead of recording the fill into its graph.
+int ensure_twiddles() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_tw_mu);
-  if (!g_tw_ready[dev]) {
+  if (g_tw_ready[dev]) return 0;
+  // (a capture elsewhere in the process does not forbid what follows: none of it
+  // touches a capturing stream)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  cudaStream_t s = nullptr;
+  e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) {
     k_twiddle_init<<<(FFT_NMAX / 2 + 255) / 256, 256, 0, s>>>();
-    const int e = cudaGetLastError();
-    if (e) return e;
-    g_tw_ready[dev] = true;
+    e = cudaGetLastError();
+    const cudaError_t done = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = done;
+    cudaStreamDestroy(s);
   }
-  return 0;
+  const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e == cudaSuccess) e = back;
+  if (e == cudaSuccess) g_tw_ready[dev] = true;
+  return e;
 }
 
 int launch_maxconv_fft(const MaxconvArgs& ma, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int te = ensure_twiddles(s);
+  const int te = ensure_twiddles();
   if (te) return te;
   const int smem = maxconv_fft_smem_bytes(ma.logN);
   const cudaError_t e = cudaFuncSetAttribute(k_maxconv_fft,
@@ -2030,7 +2045,7 @@ int long_logN(int64_t nz) {
 int launch_maxconv_long(const pn_opts* o, int64_t nx, const float* x, int64_t ny, const float* y,
                         float* z, uint8_t* p_sel, uint8_t* ws, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int e = ensure_twiddles(s);
+  int e = ensure_twiddles();
   if (e) return e;
   const int64_t nz = nx + ny - 1;
   LongArgs la;
@@ -2118,7 +2133,7 @@ TopkLayout topk_layout(int64_t batch, int64_t n, int64_t k, int n_p) {
 
 int launch_topk(const TopkArgs& ta0, uint8_t* ws, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int e = ensure_twiddles(s);
+  int e = ensure_twiddles();
   if (e) return e;
   TopkArgs ta = ta0;
   const TopkLayout L = topk_layout(ta.batch, ta.n, ta.k, ta.n_p);
