@@ -512,11 +512,10 @@ static __device__ __noinline__ float grad_factor_frexp(float acc, float x, float
 // The same, bit for bit (rounding does not depend on the scale of a mantissa),
 // for p <= 128 without a branch: with the mantissa in [0.75, 1.5) the chain stays
 // between 2^-53 and 2^75, so it is renormalised once, at the end, and the
-// exponent goes on in factors of normal powers of two, 1 but for the first unless
-// the result leaves FP32's range (a subnormal result may be rounded twice, within
-// one of its units).  About 35 instructions; with x' uniform half of the entries
-// took the renormalising loop at p = 64, some 150 instructions for every warp.
-// With the row-wise epilogue: a 2048^3 gradient GEMM in 3xTF32 185 -> 95 us.
+// exponent goes on in two factors of normal powers of two, the second 1 unless
+// the result leaves the range of normal values.  About 40 instructions; with x'
+// uniform half of the entries took the renormalising loop at p = 64, some 150
+// instructions for every warp.  With the row-wise epilogue: a 2048^3 gradient GEMM in 3xTF32 185 -> 95 us.
 __device__ __forceinline__ float grad_factor(float acc, float x, float s, int k) {
   if (k > 7) return grad_factor_frexp(acc, x, s, k);
   // s = 2^ls and x = m 2^ex; subnormal values scaled up first
@@ -535,13 +534,17 @@ __device__ __forceinline__ float grad_factor(float acc, float x, float s, int k)
   // r = m 2^(exponent - 126) with m in [0.5, 1) (k = 0: r = 1 as it is)
   const uint32_t rb = __float_as_uint(r), one = k == 0 ? 0x00800000u : 0u;
   const int e = (ex - ls) * ((1 << k) - 1) - ls + static_cast<int>((rb - one) >> 23) - 126;
-  const int e1 = min(max(e, -126), 127), e2 = min(max(e - e1, -126), 127);
-  const int e3 = max(e - e1 - e2, -126);  // below 2^-252: acc may be up to 2^127
-  float g = __fmul_rn(acc, __uint_as_float((rb & 0x007fffffu) | (0x3f000000u + one)));
-  g = __fmul_rn(__fmul_rn(g, __uint_as_float(static_cast<uint32_t>(e1 + 127) << 23)),
-                __uint_as_float(static_cast<uint32_t>(e2 + 127) << 23));
-  g = __fmul_rn(g, __uint_as_float(static_cast<uint32_t>(min(e3, 0) + 127) << 23));
-  return k > 0 && x == 0.0f ? 0.0f : g;
+  const float g = __fmul_rn(acc, __uint_as_float((rb & 0x007fffffu) | (0x3f000000u + one)));
+  // g's own exponent joins e (unless g is 0, subnormal, infinite or a NaN), so that
+  // only the last factor rounds
+  const uint32_t gb = __float_as_uint(g), eg = (gb >> 23) & 0xffu;
+  const bool plain = eg - 1u < 254u;
+  const float m = plain ? __uint_as_float((gb & 0x807fffffu) | 0x3f800000u) : g;
+  const int et = plain ? e + static_cast<int>(eg) - 127 : e;
+  const int e1 = min(max(et, -126), 127), e2 = min(max(et - e1, -126), 127);
+  const float v = __fmul_rn(__fmul_rn(m, __uint_as_float(static_cast<uint32_t>(e1 + 127) << 23)),
+                            __uint_as_float(static_cast<uint32_t>(e2 + 127) << 23));
+  return k > 0 && x == 0.0f ? acc * 0.0f : v;  // (a NaN or infinite sum is not hidden)
 }
 
 // Smallest power of two >= m (m > 0, finite); 1 for m == 0.  Returns +inf
