@@ -20,10 +20,11 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <numeric>
 #include <tuple>
-#include <vector>
 
 #include "pn_internal.h"
 #include <cuda_runtime.h>
@@ -196,11 +197,16 @@ pn_status pn_grouped_build_table(int32_t count, const int64_t* MNK, const float*
   // long contractions spread evenly and the last tiles are the cheapest, and
   // the longest strips of the image kernel start first (64 problems of 16 to
   // 1024 in BF16: 42.3 us for the persistent kernel and 36.3 for the strips,
-  // 44.4 and 38.5 in the caller's order).
-  std::vector<int32_t> order(static_cast<size_t>(count));
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int32_t x, int32_t y) { return MNK[3 * x + 2] > MNK[3 * y + 2]; });
+  // 44.4 and 38.5 in the caller's order).  Without memory for the order the table
+  // is built in the caller's: no exception may leave a C entry.
+  const std::unique_ptr<int32_t[]> order(new (std::nothrow) int32_t[static_cast<size_t>(count)]);
+  if (order) {
+    std::iota(order.get(), order.get() + count, 0);
+    std::sort(order.get(), order.get() + count, [&](int32_t x, int32_t y) {
+      const int64_t kx = MNK[3 * static_cast<int64_t>(x) + 2], ky = MNK[3 * static_cast<int64_t>(y) + 2];
+      return kx != ky ? kx > ky : x < y;
+    });
+  }
   for (int l = 0; l < 2; ++l) {
     GroupLayout& L = H->layout[l];
     L.BN = (mode == MODE_3XTF32 || l == 0) ? 128 : 256;
@@ -209,7 +215,7 @@ pn_status pn_grouped_build_table(int32_t count, const int64_t* MNK, const float*
     int64_t tiles = 0, xa = 0, xb = 0, tm = 0, tn = 0, ma = 0, mb = 0, rows = 0, cols = 0,
             words = 0, abytes = 0, bbytes = 0;
     for (int32_t slot = 0; slot < count; ++slot) {
-      const int32_t g = order[slot];
+      const int32_t g = order ? order[slot] : slot;
       const int64_t M = MNK[3 * g], N = MNK[3 * g + 1], K = MNK[3 * g + 2];
       Prob& P = probs[slot];
       std::memset(&P, 0, sizeof(P));
