@@ -11,6 +11,7 @@
 // images (recomputed from A, B, C, S_sel, p_sel rather than stored) and the
 // mask of the p values that occur; the GEMMs are the tensor-core level kernel
 // with its gradient epilogue.
+#include "pn_launch.h"
 #include "pn_pack.cuh"
 
 namespace pn {
@@ -198,13 +199,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_bw_images(const __grid_constant_
 template <int MODE>
 int launch_images_t(const BwImages& im, void* stream) {
   constexpr int smem = 128 * 129 * 4;
-  static bool done = false;
-  if (!done) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bw_images<MODE>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    done = true;
-  }
+  if (const cudaError_t e = allow_smem<k_bw_images<MODE>>(smem)) return e;
   const int blocks = im.blocks[0] + im.blocks[1] + im.blocks[2];
   if (blocks <= 0) return 0;
   const cudaError_t e = launch_pdl(k_bw_images<MODE>, dim3(blocks), dim3(BW_THREADS), smem, stream,

@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include "pn_device.cuh"
+#include "pn_launch.h"
 
 namespace pn {
 
@@ -369,8 +370,7 @@ int launch_fit(const Common& cm, const FitArgs& fa, void* stream) {
   if (ranges > 0) {
     constexpr int a_bytes = ((STREAM_K * STREAM_LD + 31) & ~31) * 4;
     const int smem = a_bytes + stages * cm.single.N * 4;
-    cudaError_t e = cudaFuncSetAttribute(k_fit_stream, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         STREAM_SMEM);
+    cudaError_t e = allow_smem<k_fit_stream>(STREAM_SMEM);
     if (e != cudaSuccess) return e;
     const int per = (cm.single.K + ranges - 1) / ranges, n = (cm.single.K + per - 1) / per;
     k_fit_stream<<<n, STREAM_THREADS, smem, s>>>(cm, fa, per, stages);

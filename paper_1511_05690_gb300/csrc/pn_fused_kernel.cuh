@@ -593,15 +593,9 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
 
 template <int MODE, int BN>
 inline int launch_fused_t(const Common& cm, const FusedArgs& fa, void* stream) {
-  static int done = 0;
   constexpr int smem = fused_smem(MODE, BN);
   static_assert(smem <= 232448, "shared memory of one CTA");
-  if (!done) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_fused_product<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    done = 1;
-  }
+  if (const cudaError_t e = allow_smem<k_fused_product<MODE, BN>>(smem)) return e;
   OperandMaps maps;
   make_raw_maps(cm, RAW_K, maps);
   const cudaError_t e = launch_pdl(k_fused_product<MODE, BN>, dim3(cm.total_tiles),

@@ -137,14 +137,9 @@ __global__ void __launch_bounds__(grouped_threads(BN, PLAIN), 1)
 template <int MODE, int BN, bool PLAIN>
 inline int launch_grouped_persist_k(const Common& cm, const GroupedRun& gr, int num_sms,
                                     void* stream) {
-  static int attr_done = 0;
-  if (!attr_done) {
-    const cudaError_t e = cudaFuncSetAttribute(k_grouped_persist<MODE, BN, PLAIN>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               smem_total(MODE, BN, 1, grouped_ng(BN, PLAIN)));
-    if (e != cudaSuccess) return e;
-    attr_done = 1;
-  }
+  if (const cudaError_t e = allow_smem<k_grouped_persist<MODE, BN, PLAIN>>(
+          smem_total(MODE, BN, 1, grouped_ng(BN, PLAIN))))
+    return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(num_sms));
   cfg.blockDim = dim3(grouped_threads(BN, PLAIN));

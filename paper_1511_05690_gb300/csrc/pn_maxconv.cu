@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "pn_device.cuh"
+#include "pn_launch.h"
 
 namespace pn {
 
@@ -1985,9 +1986,7 @@ int launch_maxconv_fft(const MaxconvArgs& ma, void* stream) {
   const int te = ensure_twiddles();
   if (te) return te;
   const int smem = maxconv_fft_smem_bytes(ma.logN);
-  const cudaError_t e = cudaFuncSetAttribute(k_maxconv_fft,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  if (const cudaError_t e = allow_smem<k_maxconv_fft>(maxconv_fft_smem_bytes(FFT_LOG_NMAX))) return e;
   // eight values per thread: several CTAs per SM on short problems
   const int N = 1 << ma.logN;
   const int threads = N / 8 < 64 ? 64 : N / 8;
@@ -2002,9 +2001,7 @@ int maxconv_exact_smem_bytes() {
 int launch_maxconv_exact(const MaxconvArgs& ma, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int smem = maxconv_exact_smem_bytes();
-  const cudaError_t e = cudaFuncSetAttribute(k_maxconv_exact,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  if (const cudaError_t e = allow_smem<k_maxconv_exact>(smem)) return e;
   const int iblocks = (ma.nx + MCX_IB - 1) / MCX_IB;
   if (iblocks > 1) {  // partial maxima meet in z by atomicMax: start from 0
     const cudaError_t me = cudaMemset2DAsync(ma.z, sizeof(float) * ma.ldz, 0,
@@ -2075,14 +2072,13 @@ int launch_maxconv_long(const pn_opts* o, int64_t nx, const float* x, int64_t ny
       la, reinterpret_cast<double2*>(ws + L.off_tlo), reinterpret_cast<double2*>(ws + L.off_thi));
   if ((e = cudaGetLastError())) return e;
   const int N1 = 1 << la.l1, N2 = 1 << la.l2;
-  const int smem_col = (LONG_CC * (N1 + 2) + N1 / 2) * static_cast<int>(sizeof(double2));
-  const int smem_row = (N2 + N2 / 2) * static_cast<int>(sizeof(double2));
-  if ((e = cudaFuncSetAttribute(k_long_col_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col)))
-    return e;
-  if ((e = cudaFuncSetAttribute(k_long_col_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col)))
-    return e;
-  if ((e = cudaFuncSetAttribute(k_long_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_row)))
-    return e;
+  const auto col_bytes = [](int n) { return (LONG_CC * (n + 2) + n / 2) * static_cast<int>(sizeof(double2)); };
+  const auto row_bytes = [](int n) { return (n + n / 2) * static_cast<int>(sizeof(double2)); };
+  const int smem_col = col_bytes(N1), smem_row = row_bytes(N2);
+  constexpr int MAX_N1 = 1 << 10, MAX_N2 = 1 << 12;  // N = 2^22
+  if ((e = allow_smem<k_long_col_fwd>(col_bytes(MAX_N1)))) return e;
+  if ((e = allow_smem<k_long_col_inv>(col_bytes(MAX_N1)))) return e;
+  if ((e = allow_smem<k_long_rows>(row_bytes(MAX_N2)))) return e;
   const dim3 cols(N2 / LONG_CC), col_threads(LONG_CC * N1 / 8);
   cudaLaunchConfig_t rows = {};
   rows.gridDim = dim3(N1);
@@ -2145,12 +2141,10 @@ int launch_topk(const TopkArgs& ta0, uint8_t* ws, void* stream) {
   ta.diag = reinterpret_cast<int32_t*>(ws + L.off_diag);
   const int N = 1 << ta.logN;
   const int smem_sums = (N + N / 2) * static_cast<int>(sizeof(double2));
-  if ((e = cudaFuncSetAttribute(k_topk_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_sums)))
+  if ((e = allow_smem<k_topk_sums>((FFT_NMAX + FFT_NMAX / 2) * static_cast<int>(sizeof(double2)))))
     return e;
   const int nb = (ta.nz + 31) / 32;
-  const int smem_pop = nb * 8;
-  if ((e = cudaFuncSetAttribute(k_topk_pop, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pop)))
-    return e;
+  const int smem_pop = nb * 8;  // at most 2 KB
   // threads: two groups of eight values each in the first pass; as many CTAs
   // as fit on the SMs, each with a run of the work items
   const int threads = N / 16 < 64 ? 64 : N / 16 > FFT_THREADS ? FFT_THREADS : N / 16;
@@ -2162,8 +2156,7 @@ int launch_topk(const TopkArgs& ta0, uint8_t* ws, void* stream) {
   k_topk_sums<<<static_cast<unsigned>(items < room ? items : room), threads, smem_sums, s>>>(ta);
   if (ta.k <= TOPK_KMAX) {
     const int smem = topk_merge_smem(ta.nz, ta.k);
-    if ((e = cudaFuncSetAttribute(k_topk_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
-      return e;
+    if ((e = allow_smem<k_topk_merge>(topk_merge_smem(FFT_NMAX - 1, TOPK_KMAX)))) return e;
     k_topk_merge<<<2 * ta.batch, TOPK_THREADS, smem, s>>>(ta);
   } else {
     k_topk_first<<<2 * ta.batch, FFT_THREADS, 0, s>>>(ta);

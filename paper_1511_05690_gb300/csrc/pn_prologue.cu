@@ -16,7 +16,7 @@
 #include <cuda_fp8.h>
 
 #include "pn_image.cuh"
-#include "pn_split.h"
+#include "pn_launch.h"
 
 namespace pn {
 
@@ -644,13 +644,7 @@ int launch_tma_t(const Common& cm, const Level& lv, void* stream, const OperandM
   using CA = TmaCfg<MODE, false>;
   using CB = TmaCfg<MODE, true>;
   constexpr int smem = CA::SMEM > CB::SMEM ? CA::SMEM : CB::SMEM;
-  static bool attr_done = false;
-  if (!attr_done) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_image_tma<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
+  if (const cudaError_t e = allow_smem<k_image_tma<MODE>>(smem)) return e;
   static_assert(CA::CTAS == TMA_CTAS_32K && CB::CTAS == TMA_CTAS_32K, "see tma_together");
   // the resident CTAs, shared out by the operands' tiles
   const int grid = tma_ctas(xa + xb);
@@ -726,13 +720,7 @@ bool encode_fp32_2d(TensorMapBytes& out, const float* base, int64_t rows, int64_
 template <int MODE>
 int launch_power_t(const Common& cm, const Level& lv, void* stream, int xa, int xb) {
   const int smem = xb > 0 ? mode_bk(MODE) * 129 * 4 : 0;
-  static bool attr_done = false;
-  if (!attr_done) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_power<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, mode_bk(MODE) * 129 * 4);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
+  if (const cudaError_t e = allow_smem<k_power<MODE>>(mode_bk(MODE) * 129 * 4)) return e;
   const int n_a = lv.is_top ? xa : lower_grid(xa, img_min_blocks<MODE>());
   const int n_b = lv.is_top ? xb : lower_grid(xb, img_min_blocks<MODE>());
   const cudaError_t e =
@@ -1043,13 +1031,7 @@ __global__ void __launch_bounds__(PRO_THREADS)
 template <int MODE>
 int launch_strips_t(const Common& cm, const Level& lv, void* stream) {
   constexpr int smem = strip_smem<MODE>();
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_strips<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
+  if (const cudaError_t e = allow_smem<k_strips<MODE>>(smem)) return e;
   const int n_a = cm.total_tm, n_b = cm.total_tn * (cm.BN / TILE_M);
   const cudaError_t e = launch_pdl(k_strips<MODE>, dim3(4 * (n_a + n_b)), dim3(PRO_THREADS), smem,
                                    stream, cm, lv, n_a, n_b);

@@ -1,6 +1,7 @@
 // Host arithmetic of the launches, free of CUDA.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 namespace pn {
@@ -21,5 +22,18 @@ inline int image_split(int64_t xa, int64_t xb, int ctas) {
   const int64_t hi = std::min<int64_t>(below + 1, ctas - 1);
   return static_cast<int>(worst(hi) < worst(lo) ? hi : lo);
 }
+
+// The devices (0 .. 63) for which something has been done once; safe between threads.
+class DeviceSet {
+ public:
+  bool has(int dev) const { return known(dev) && (bits_.load(std::memory_order_acquire) >> dev) & 1u; }
+  void add(int dev) {
+    if (known(dev)) bits_.fetch_or(uint64_t(1) << dev, std::memory_order_release);
+  }
+
+ private:
+  static bool known(int dev) { return dev >= 0 && dev < 64; }
+  std::atomic<uint64_t> bits_{0};
+};
 
 }  // namespace pn

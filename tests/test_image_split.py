@@ -19,12 +19,22 @@ def split(tmp_path_factory):
     d = tmp_path_factory.mktemp("split")
     (d / "s.cpp").write_text(
         '#include "pn_split.h"\n'
-        'extern "C" int split(long long a, long long b, int n) { return pn::image_split(a, b, n); }\n')
+        'extern "C" int split(long long a, long long b, int n) { return pn::image_split(a, b, n); }\n'
+        'static pn::DeviceSet set;\n'
+        'extern "C" int add(int d) { int had = set.has(d); set.add(d); return had; }\n')
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "s.cpp"),
                     "-o", str(d / "s.so")], check=True)
     f = ctypes.CDLL(str(d / "s.so")).split
     f.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
+    f.lib = str(d / "s.so")
     return f
+
+
+def test_what_is_done_once_per_device(split):
+    # a kernel's shared-memory limit belongs to a device: each of two needs its own, and
+    # one beyond the set's is never taken for done
+    add = ctypes.CDLL(split.lib).add
+    assert [add(d) for d in (0, 0, 1, 1, 63, 63, 64, 64, -1, -1)] == [0, 1, 0, 1, 0, 1, 0, 0, 0, 0]
 
 
 def _worst(xa, xb, n, ctas):
