@@ -80,8 +80,12 @@ def check_device_status(device, where: str) -> None:
 def _stream_ptr(stream):
     if stream is None:
         # the current stream's handle without building its Python object, which
-        # took 3 of the 20 us of host time of a small product
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # took 3 of the 20 us of host time of a small product; by the public call
+        # where torch has the private one no more
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return ctypes.c_void_p(raw(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
 
