@@ -343,17 +343,23 @@ Level make_level(const Layout& L, const pn_opts* o, uint8_t* ws, const Schedule&
 
 // Tile width of the one-launch product (k_fused_product), 0 for the level
 // launches.  It takes outputs of at most one tile per SM (128 x 64, or 128 x
-// 128) whose build time per level, 32 columns of K at a time, stays below
-// FUSED_NS: the level launches' images are built once per operand block over
-// all SMs, so they win on long contractions, but a call of theirs is 23
-// launches, about 100 us with their host time.  Nanoseconds per 32 columns,
-// maxima and one level, at 64 / 128 wide tiles (measured, K = 1024 .. 2048):
-// tensor copies (16-byte aligned rows): 3xTF32 1450 / 2010, 16-bit 1020 / 1080,
-// E4M3 1150 / 1460; unaligned rows: 2130 / 4050, 1700 / 2710, 1980 / 3420; TF32
-// as 3xTF32.  Level launches -> one launch: 256^3 3xTF32 (P = {1..128}) 94 -> 30
-// us, 512^3 117 -> 35, 1024^3 99 -> 58, 1024 x 2048 x 1536 BF16 92 -> 66, the
-// 512-vertex closure 1712 -> 1055.
-constexpr int64_t FUSED_NS = 55000;
+// 128) up to a contraction that depends on the format, the width and whether
+// rows are 16-byte aligned (tensor copies, or 4-byte ones): it pays for its
+// operands once per tile and level, the level launches once per operand block
+// over all SMs, but 3.5 us of host time per launch (16 of them, about 75 us).
+// The limits are where the two take the same time, on uniform data (one level)
+// or on data that opens every level of P = {1..64}, whichever comes first; in
+// us, one launch / level launches, 1000 x 1000 (64 wide) and 1400 x 1408 (128):
+//              one level        every level
+//   3xTF32  64 aligned  K = 1024  70 / 82    402 / 422   (1152: 76 / 85, 435 / 434)
+//                       512       45 / 75    258 / 353
+//           64 else     768       72 / 83    393 / 408
+//           128 aligned 256       54 / 80    324 / 288
+//   BF16    64 aligned  1024      51 / 77    274 / 286
+//           128 aligned 512       38 / 75    239 / 243
+//   E4M3    64 aligned  512      127 / 150   172 / 187   (1024: 187 / 150, 265 / 176)
+//           64 else     384      151 / 182   217 / 240
+//           128 aligned 256      149 / 133   185 / 181
 int fused_bn(const pn_opts* o, int64_t M, int64_t N, int64_t K, bool aligned, int sms) {
   if (o->tile_m || o->tile_n || o->scaling == 1 || o->correction == 2 || o->estimator == 2 ||
       (o->debug_flags & ~16) || host_tuned_bn(o->compute, M, N, K))
@@ -361,12 +367,17 @@ int fused_bn(const pn_opts* o, int64_t M, int64_t N, int64_t K, bool aligned, in
   const int64_t rows = ceil_div(M, TILE_M);
   const int bn = rows * ceil_div(N, 64) <= sms ? 64 : rows * ceil_div(N, 128) <= sms ? 128 : 0;
   if (bn == 0) return 0;
-  const int kind = o->compute == PN_F32_EXACT || o->compute == PN_TF32 ? 0
-                   : o->compute == PN_E4M3                             ? 2
-                                                                       : 1;
-  constexpr int ns[2][3][2] = {{{2130, 4050}, {1700, 2710}, {1980, 3420}},
-                               {{1450, 2010}, {1020, 1080}, {1150, 1460}}};
-  return ceil_div(K, 32) * ns[aligned ? 1 : 0][kind][bn == 128 ? 1 : 0] <= FUSED_NS ? bn : 0;
+  // the longest contraction: 64 and 128 wide, else and aligned
+  struct Limits { int k64[2], k128[2]; };
+  constexpr Limits f32 = {{768, 1024}, {128, 192}}, tf32 = {{896, 1152}, {128, 192}},
+                   bf16 = {{768, 1024}, {320, 512}}, f16 = {{768, 896}, {320, 512}},
+                   e4m3 = {{384, 512}, {128, 128}};
+  const Limits& l = o->compute == PN_F32_EXACT ? f32
+                    : o->compute == PN_TF32    ? tf32
+                    : o->compute == PN_BF16    ? bf16
+                    : o->compute == PN_F16     ? f16
+                                               : e4m3;
+  return K <= (bn == 64 ? l.k64 : l.k128)[aligned ? 1 : 0] ? bn : 0;
 }
 
 // The product proper, arguments already checked.

@@ -11,8 +11,8 @@
 //      complete;
 //   3. the level kernel's epilogue on the tile; entries left take the CTA to
 //      the next level.  Tiles never wait on one another.
-// The level launches (maxima, two image kernels and a GEMM per level) cost
-// about 1.3 us on the GPU and 3.5 us on the host each, 94 us for a 256^3
+// The level launches (maxima, and an image kernel and a GEMM per level) cost
+// about 1.3 us on the GPU and 3.5 us on the host each, 78 us for a 256^3
 // product whose work takes a few; their images are built once per operand
 // block, here once per tile.  What bounds this kernel is that building: about
 // 270 instructions per warp and block of 32 columns in 3xTF32 and a barrier
