@@ -142,11 +142,7 @@ __global__ void __launch_bounds__(FIT_THREADS)
 // bound per SM (about 4.7 clocks each: 136 us for 1024 samples at n = 8192); here
 // B is read once: 67 us, and 24 for the merge.  The partial sums go to
 // part[x][value][sample].
-constexpr int STREAM_THREADS = 1024;
-constexpr int STREAM_K = 16;                      // contraction indices of A per load
-constexpr int STREAM_LD = STREAM_THREADS + 1;     // floats between them
-constexpr int STREAM_MAX_STAGES = 4;
-
+// (STREAM_K indices of A per load, STREAM_LD floats between them.)
 __global__ void __launch_bounds__(STREAM_THREADS, 1)
     k_fit_stream(const __grid_constant__ Common cm, const __grid_constant__ FitArgs fa, int per,
                  int stages) {
@@ -157,7 +153,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 1)
   const int s = threadIdx.x, lane = s & 31, warp = s >> 5;
   const int row_floats = P.N;
   float* const as = reinterpret_cast<float*>(sm_fit);  // [STREAM_K][STREAM_LD]
-  float* const ring = as + ((STREAM_K * STREAM_LD + 31) & ~31);
+  float* const ring = as + STREAM_A_FLOATS;
   const int k0 = blockIdx.x * per, k1 = min(P.K, k0 + per);
   const int i = s < fa.n_fit ? fa.fi[s] : 0, j = s < fa.n_fit ? fa.fj[s] : 0;
   const bool valid = s < fa.n_fit && i >= 0 && i < P.M && j >= 0 && j < P.N;
@@ -339,40 +335,20 @@ __global__ void k_fit_solve(const __grid_constant__ FitArgs fa) {
 
 }  // namespace
 
-// Ranges of the contraction for k_fit_stream (0: k_fit_samples) and the stages of
-// its ring.  It needs whole aligned rows of B, a thread per sample and room for
-// the partial sums, and reads all of B where k_fit_samples reads a sector per
-// term: B's rows at the copy rate cost less up to about 26 columns per sample
-// (1024 samples, in us, stream with merge against a block per sample: n = 16384
-// 246 / 285, 8192 91 / 136, 4096 63 / 70); below 4 M terms the merge costs more than the
-// scattered reads.
-constexpr int STREAM_SMEM = 220 * 1024;
-static int fit_ranges(const Common& cm, const FitArgs& fa, int* stages) {
-  const Prob& P = cm.single;
-  constexpr int a_bytes = ((STREAM_K * STREAM_LD + 31) & ~31) * 4;
-  if (fa.n_fit > STREAM_THREADS || (int64_t)fa.n_fit * P.K < (4 << 20) || P.N > 16 * fa.n_fit)
-    return 0;
-  if ((P.N & 3) || (P.ldb & 3) || (reinterpret_cast<uintptr_t>(P.B) & 15)) return 0;
-  const int n = (STREAM_SMEM - a_bytes) / (P.N * 4);
-  if (n < 2) return 0;
-  *stages = n < STREAM_MAX_STAGES ? n : STREAM_MAX_STAGES;
-  const int64_t room = fa.part_floats / ((int64_t)(fa.n_p + 1) * fa.n_fit);
-  int ranges = host_device_sms();
-  if (ranges > P.K / STREAM_K) ranges = P.K / STREAM_K;
-  if (ranges > room) ranges = static_cast<int>(room);
-  return ranges < 16 ? 0 : ranges;
-}
-
 int launch_fit(const Common& cm, const FitArgs& fa, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const Prob& P = cm.single;
+  const bool whole_rows = (P.N & 3) == 0 && (P.ldb & 3) == 0 &&
+                          (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
   int stages = 0;
-  const int ranges = fit_ranges(cm, fa, &stages);
+  const int ranges = whole_rows ? fit_stream_ranges(P.N, P.K, fa.n_fit, fa.n_p, fa.part_floats,
+                                                    host_device_sms(), &stages)
+                                : 0;
   if (ranges > 0) {
-    constexpr int a_bytes = ((STREAM_K * STREAM_LD + 31) & ~31) * 4;
-    const int smem = a_bytes + stages * cm.single.N * 4;
+    const int smem = 4 * (STREAM_A_FLOATS + stages * P.N);
     cudaError_t e = allow_smem<k_fit_stream>(STREAM_SMEM);
     if (e != cudaSuccess) return e;
-    const int per = (cm.single.K + ranges - 1) / ranges, n = (cm.single.K + per - 1) / per;
+    const int per = (P.K + ranges - 1) / ranges, n = (P.K + per - 1) / per;
     k_fit_stream<<<n, STREAM_THREADS, smem, s>>>(cm, fa, per, stages);
     k_fit_merge<<<(fa.n_fit + MERGE_SAMPLES - 1) / MERGE_SAMPLES, 32 * MERGE_WARPS, 0, s>>>(cm, fa, n);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

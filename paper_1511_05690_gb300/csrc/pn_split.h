@@ -23,6 +23,33 @@ inline int image_split(int64_t xa, int64_t xb, int ctas) {
   return static_cast<int>(worst(hi) < worst(lo) ? hi : lo);
 }
 
+// The affine fit's stream over B's rows (k_fit_stream): a thread per sample, the
+// samples' values of A for STREAM_K indices at a time, a ring of whole rows of B.
+constexpr int STREAM_THREADS = 1024;
+constexpr int STREAM_K = 16;
+constexpr int STREAM_LD = STREAM_THREADS + 1;
+constexpr int STREAM_A_FLOATS = (STREAM_K * STREAM_LD + 31) & ~31;
+constexpr int STREAM_MAX_STAGES = 4;
+constexpr int STREAM_SMEM = 220 * 1024;
+
+// Ranges of the contraction for the stream (0: k_fit_samples) and the stages of its
+// ring, where B's rows are 16-byte aligned and N a multiple of 4.  It needs a thread
+// per sample and room for the partial sums (part_floats), and reads all of B where
+// k_fit_samples reads a sector per term: B's rows at the copy rate cost less up to
+// about 26 columns per sample (1024 samples, in us, stream with merge against a
+// block per sample: n = 16384 246 / 285, 8192 91 / 136, 4096 63 / 70); below 4 M terms
+// the merge costs more than the scattered reads.
+inline int fit_stream_ranges(int64_t N, int64_t K, int64_t n_fit, int n_p, int64_t part_floats,
+                             int sms, int* stages) {
+  if (n_fit > STREAM_THREADS || n_fit * K < (4 << 20) || N > 16 * n_fit) return 0;
+  const int64_t n = (STREAM_SMEM / 4 - STREAM_A_FLOATS) / N;
+  if (n < 2) return 0;
+  *stages = static_cast<int>(std::min<int64_t>(n, STREAM_MAX_STAGES));
+  const int64_t room = part_floats / ((n_p + 1) * n_fit);
+  const int64_t ranges = std::min<int64_t>(std::min<int64_t>(sms, K / STREAM_K), room);
+  return ranges < 16 ? 0 : static_cast<int>(ranges);
+}
+
 // The devices (0 .. 63) for which something has been done once; safe between threads.
 class DeviceSet {
  public:

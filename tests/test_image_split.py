@@ -20,6 +20,8 @@ def split(tmp_path_factory):
     (d / "s.cpp").write_text(
         '#include "pn_split.h"\n'
         'extern "C" int split(long long a, long long b, int n) { return pn::image_split(a, b, n); }\n'
+        'extern "C" int ranges(long long N, long long K, long long f, int n_p, long long room) {\n'
+        '  int stages = 0; return pn::fit_stream_ranges(N, K, f, n_p, room, 152, &stages); }\n'
         'static pn::DeviceSet set;\n'
         'extern "C" int add(int d) { int had = set.has(d); set.add(d); return had; }\n')
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "s.cpp"),
@@ -35,6 +37,19 @@ def test_what_is_done_once_per_device(split):
     # one beyond the set's is never taken for done
     add = ctypes.CDLL(split.lib).add
     assert [add(d) for d in (0, 0, 1, 1, 63, 63, 64, 64, -1, -1)] == [0, 1, 0, 1, 0, 1, 0, 0, 0, 0]
+
+
+def test_the_affine_fit_streams_where_its_tests_mean_it_to(split):
+    from test_gpu_fit_stream_sums import CASES
+    ranges = ctypes.CDLL(split.lib).ranges
+    ranges.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int, ctypes.c_longlong]
+    for M, N, K, n_fit, p_log2, _ in CASES:
+        got = ranges(N, K, n_fit, len(p_log2), M * (-(-N // 32)))  # the least state array
+        assert 16 <= got <= 152 and got * 16 <= K and N % 4 == 0, (M, N, K, got)
+    # too few terms, too many columns per sample, no room, more samples than threads
+    for N, K, f, room in ((4096, 4095, 1024, 1 << 30), (16388, 8192, 1024, 1 << 30),
+                          (4096, 8192, 1024, 15 * 8 * 1024), (4096, 8192, 1025, 1 << 30)):
+        assert ranges(N, K, f, 7, room) == 0
 
 
 def _worst(xa, xb, n, ctas):
