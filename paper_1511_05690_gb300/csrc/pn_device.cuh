@@ -438,8 +438,8 @@ __host__ __device__ __forceinline__ uint32_t sw128_offset(uint32_t r, uint32_t b
   return r * 128u + ((((b >> 4) ^ (r & 7u)) & 7u) << 4) + (b & 15u);
 }
 
-// Two FP32 values in one register pair, and their products in one instruction
-// (each rounded as by itself).
+// Two FP32 values in one register pair; their products, sums and fused products
+// in one instruction (each rounded as by itself).
 __device__ __forceinline__ uint64_t f32x2_pack(float a, float b) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -451,6 +451,16 @@ __device__ __forceinline__ void f32x2_unpack(uint64_t v, float& a, float& b) {
 __device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
 

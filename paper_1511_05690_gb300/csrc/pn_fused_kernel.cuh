@@ -267,22 +267,6 @@ __device__ __forceinline__ void sts_u4(uint32_t addr, uint4 v) {
                : "memory");
 }
 
-// Values are held as pairs: mul.rn.f32x2 makes two of the squarings (each
-// rounded as by itself) in one issue slot.
-__device__ __forceinline__ uint64_t pair2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpair2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // The MMAs of one image block (128 bytes of K): K steps of 32 bytes, 3xTF32 as
 // lo hi + hi lo + hi hi (small terms first), the order of run_mma.
 template <int MODE, int BN>
@@ -310,8 +294,8 @@ __device__ __forceinline__ void fused_mma(uint32_t acc, uint32_t sa, uint32_t sb
 // x / s for scales whose reciprocal is no normal float.
 static __device__ __noinline__ uint64_t div2(uint64_t v, float s) {
   float a, b;
-  unpair2(v, a, b);
-  return pair2(a / s, b / s);
+  f32x2_unpack(v, a, b);
+  return f32x2_pack(a / s, b / s);
 }
 
 // Scales and powers U chunks of EPC values.  inv: the scales' reciprocals, or
@@ -323,14 +307,14 @@ __device__ __forceinline__ void fused_scale(uint64_t (&v)[U][E2], const float (&
   for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int e = 0; e < E2; ++e)
-      v[u][e] = exact ? mul2(v[u][e], pair2(inv[u], inv[u])) : div2(v[u][e], inv[u]);
+      v[u][e] = exact ? f32x2_mul(v[u][e], f32x2_pack(inv[u], inv[u])) : div2(v[u][e], inv[u]);
 }
 template <int U, int E2>
 __device__ __forceinline__ void fused_times(uint64_t (&v)[U][E2], bool square, float f) {
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int e = 0; e < E2; ++e) v[u][e] = mul2(v[u][e], square ? v[u][e] : pair2(f, f));
+    for (int e = 0; e < E2; ++e) v[u][e] = f32x2_mul(v[u][e], square ? v[u][e] : f32x2_pack(f, f));
 }
 
 // Casts and stores U chunks at the image addresses dst[u] + at (3xTF32: the lo
@@ -345,7 +329,7 @@ __device__ __forceinline__ void fused_store(const uint32_t (&dst)[U], uint32_t s
   for (int u = 0; u < U; ++u) {
     float f[EPC];
 #pragma unroll
-    for (int e = 0; e < EPC / 2; ++e) unpair2(v[u][e], f[2 * e], f[2 * e + 1]);
+    for (int e = 0; e < EPC / 2; ++e) f32x2_unpack(v[u][e], f[2 * e], f[2 * e + 1]);
     uint4 hi, lo;
     PK::pack(f, hi, lo);
     const uint32_t d = (dst[u] ^ sx) + at;
@@ -530,7 +514,7 @@ __global__ void __launch_bounds__(FUSED_BUILD, 1)
               const uint32_t b0 = blk + src_b[u];
 #pragma unroll
               for (int e = 0; e < EPC; e += 2)
-                vb[u][e / 2] = pair2(lds_f32(b0 + e * BN * 4), lds_f32(b0 + (e + 1) * BN * 4));
+                vb[u][e / 2] = f32x2_pack(lds_f32(b0 + e * BN * 4), lds_f32(b0 + (e + 1) * BN * 4));
             }
           }
           if (do_a && do_b) {  // their chains of squarings interleaved

@@ -108,7 +108,7 @@ __device__ __forceinline__ void div_scales(float (&v)[U][EPC], const float (&s)[
 
 // v <- v^p * opscale with p = 2^plog, or p = 1.5 * 2^plog for a half level
 // (y * sqrt(y), y = v^(2^plog)); the squarings of all U x EPC values
-// interleaved (independent chains; the same products as pow2k value by value),
+// interleaved (independent chains; the same products as value by value),
 // two per instruction: the strips of grouped products run out of issue slots.
 template <int U, int EPC>
 __device__ __forceinline__ void power_all(float (&v)[U][EPC], int plog, int half, float opscale) {

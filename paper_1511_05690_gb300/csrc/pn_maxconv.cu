@@ -209,47 +209,27 @@ __device__ __forceinline__ int slot(int i) { return i ^ (((i >> 4) & 3) << 1); }
 struct alignas(16) cff {
   uint64_t h, l;
 };
-__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
 __device__ __forceinline__ float2 f2_unpack(uint64_t v) {
   float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  f32x2_unpack(v, r.x, r.y);
   return r;
 }
 constexpr uint64_t F2_NEG = 0xbf800000bf800000ull;  // (-1, -1)
-__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) { return f2_fma(b, F2_NEG, a); }
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) { return f32x2_fma(b, F2_NEG, a); }
 __device__ __forceinline__ uint64_t f2_neg(uint64_t a) { return a ^ 0x8000000080000000ull; }
 
 // a + b: the rounding error of the high parts by Knuth's two-sum, the low parts
 // added to it (not renormalised).
 __device__ __forceinline__ cff ff_add(uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl) {
-  const uint64_t s = f2_add(ah, bh), t = f2_sub(s, ah);
-  const uint64_t e = f2_add(f2_sub(ah, f2_sub(s, t)), f2_sub(bh, t));
-  return cff{s, f2_add(e, f2_add(al, bl))};
+  const uint64_t s = f32x2_add(ah, bh), t = f2_sub(s, ah);
+  const uint64_t e = f32x2_add(f2_sub(ah, f2_sub(s, t)), f2_sub(bh, t));
+  return cff{s, f32x2_add(e, f32x2_add(al, bl))};
 }
 // a - b
 __device__ __forceinline__ cff ff_sub(uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl) {
   const uint64_t s = f2_sub(ah, bh), t = f2_sub(s, ah);
-  const uint64_t e = f2_sub(f2_sub(ah, f2_sub(s, t)), f2_add(bh, t));
-  return cff{s, f2_add(e, f2_sub(al, bl))};
+  const uint64_t e = f2_sub(f2_sub(ah, f2_sub(s, t)), f32x2_add(bh, t));
+  return cff{s, f32x2_add(e, f2_sub(al, bl))};
 }
 
 __device__ __forceinline__ double2 c_add(double2 a, double2 b) {
@@ -276,7 +256,7 @@ __device__ __forceinline__ cff c_conj(cff a) {
 // i a = (-y, x)
 __device__ __forceinline__ cff c_muli(cff a) {
   const float2 h = f2_unpack(a.h), l = f2_unpack(a.l);
-  return cff{f2_pack(-h.y, h.x), f2_pack(-l.y, l.x)};
+  return cff{f32x2_pack(-h.y, h.x), f32x2_pack(-l.y, l.x)};
 }
 __device__ __forceinline__ cff c_add_conj(cff a, cff b) { return c_add(a, c_conj(b)); }
 __device__ __forceinline__ cff c_sub_conj(cff a, cff b) { return c_sub(a, c_conj(b)); }
@@ -289,12 +269,12 @@ __device__ __forceinline__ cff c_mul_mi(cff a) {
 __device__ __forceinline__ cff cmul(cff w, cff v) {
   const cff iw = c_muli(w);
   const float2 vh = f2_unpack(v.h), vl = f2_unpack(v.l);
-  const uint64_t xh = f2_pack(vh.x, vh.x), xl = f2_pack(vl.x, vl.x);
-  const uint64_t yh = f2_pack(vh.y, vh.y), yl = f2_pack(vl.y, vl.y);
-  const uint64_t p = f2_mul(xh, w.h), q = f2_mul(yh, iw.h);
-  uint64_t e = f2_fma(xh, w.h, f2_neg(p)), f = f2_fma(yh, iw.h, f2_neg(q));
-  e = f2_fma(xh, w.l, f2_fma(xl, w.h, e));
-  f = f2_fma(yh, iw.l, f2_fma(yl, iw.h, f));
+  const uint64_t xh = f32x2_pack(vh.x, vh.x), xl = f32x2_pack(vl.x, vl.x);
+  const uint64_t yh = f32x2_pack(vh.y, vh.y), yl = f32x2_pack(vl.y, vl.y);
+  const uint64_t p = f32x2_mul(xh, w.h), q = f32x2_mul(yh, iw.h);
+  uint64_t e = f32x2_fma(xh, w.h, f2_neg(p)), f = f32x2_fma(yh, iw.h, f2_neg(q));
+  e = f32x2_fma(xh, w.l, f32x2_fma(xl, w.h, e));
+  f = f32x2_fma(yh, iw.l, f32x2_fma(yl, iw.h, f));
   return ff_add(p, e, q, f);
 }
 __device__ __forceinline__ cff cmulc(cff w, cff v) { return cmul(c_conj(w), v); }
@@ -715,7 +695,7 @@ __global__ void __launch_bounds__(MC_THREADS, 1)
     for (int k = tid; k < N; k += nt) {
       const float xr = k < ma.nx ? pow_f32(x[k] * isx, plog) : 0.0f;
       const float yr = k < ma.ny ? pow_f32(y[k] * isy, plog) : 0.0f;
-      a[slot(k)] = cff{f2_pack(xr, yr), 0ull};
+      a[slot(k)] = cff{f32x2_pack(xr, yr), 0ull};
       sq = fmaf(xr, xr, fmaf(yr, yr, sq));
       large_x += xr >= least;
       large_y += yr >= least;

@@ -10,13 +10,6 @@
 
 namespace pn {
 
-// x^(2^plog) by repeated squaring (each step one correctly rounded multiply).
-__device__ __forceinline__ float pow2k(float x, int plog) {
-#pragma unroll 1
-  for (int t = 0; t < plog; ++t) x = x * x;
-  return x;
-}
-
 __device__ __forceinline__ uint32_t tf32_bits(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
