@@ -1316,7 +1316,7 @@ __global__ void __launch_bounds__(LONG_THREADS, 2)
   const double sxy = scale;
   const double inv4n = __hiloint2double((1023 - 2 - la.logN) << 20, 0);  // 1 / (4 N)
   const int plog = la.p_log2[q];
-  unsigned long long terms = 0ull;
+  unsigned terms = 0u;  // at most 8 x 2^21, 2^29 in a warp
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const int m = (r * ng + rg) * N2 + n2;
@@ -1327,10 +1327,13 @@ __global__ void __launch_bounds__(LONG_THREADS, 2)
       la.z[m] = static_cast<float>(sxy * root_pow2(S, plog));
       la.res[m] = static_cast<uint8_t>(plog | (stable ? 0 : 0x80));
     } else {
-      terms += static_cast<unsigned long long>(terms_of(m, la.nx, la.ny));
+      terms += static_cast<unsigned>(terms_of(m, la.nx, la.ny));
     }
   }
-  if (terms) atomicAdd(la.open_terms + q, terms);
+  // one atomic per warp (one per thread, all on one address: 5 us more for a level
+  // of 2^19 with every index open)
+  terms = __reduce_add_sync(0xffffffffu, terms);
+  if ((tid & 31) == 0 && terms) atomicAdd(la.open_terms + q, static_cast<unsigned long long>(terms));
 }
 
 // After level q: nothing open ends the call; few open terms are summed
@@ -2054,15 +2057,20 @@ int launch_maxconv_long(const pn_opts* o, int64_t nx, const float* x, int64_t ny
   const int N1 = 1 << la.l1, N2 = 1 << la.l2;
   const auto col_bytes = [](int n) { return (LONG_CC * (n + 2) + n / 2) * static_cast<int>(sizeof(double2)); };
   const auto row_bytes = [](int n) { return (n + n / 2) * static_cast<int>(sizeof(double2)); };
-  const int smem_col = col_bytes(N1), smem_row = row_bytes(N2);
-  constexpr int MAX_N1 = 1 << 10, MAX_N2 = 1 << 12;  // N = 2^22
-  if ((e = allow_smem<k_long_col_fwd>(col_bytes(MAX_N1)))) return e;
-  if ((e = allow_smem<k_long_col_inv>(col_bytes(MAX_N1)))) return e;
-  if ((e = allow_smem<k_long_rows>(row_bytes(MAX_N2)))) return e;
-  const dim3 cols(N2 / LONG_CC), col_threads(LONG_CC * N1 / 8);
+  const int col_threads = LONG_CC * N1 / 8, row_threads = N2 / 8 < 32 ? 32 : N2 / 8;
+  const dim3 cols(N2 / LONG_CC);
+  const int sms = host_device_sms();
+  const int smem_col = even_share_smem(col_bytes(N1), N2 / LONG_CC, col_threads, sms);
+  const int smem_row = even_share_smem(row_bytes(N2), N1, row_threads, sms);
+  constexpr int DIRECT_CTAS = 152 * 4, DIRECT_THREADS = 256;
+  const int smem_direct = even_share_smem(0, DIRECT_CTAS, DIRECT_THREADS, sms);
+  if ((e = allow_smem<k_long_col_fwd>(CTA_SMEM_MAX))) return e;
+  if ((e = allow_smem<k_long_col_inv>(CTA_SMEM_MAX))) return e;
+  if ((e = allow_smem<k_long_rows>(CTA_SMEM_MAX))) return e;
+  if ((e = allow_smem<k_long_direct>(CTA_SMEM_MAX))) return e;
   cudaLaunchConfig_t rows = {};
   rows.gridDim = dim3(N1);
-  rows.blockDim = dim3(N2 / 8 < 32 ? 32 : N2 / 8);
+  rows.blockDim = dim3(row_threads);
   rows.dynamicSmemBytes = smem_row;
   rows.stream = s;
   cudaLaunchAttribute attr[2];
@@ -2075,10 +2083,11 @@ int launch_maxconv_long(const pn_opts* o, int64_t nx, const float* x, int64_t ny
   rows.attrs = attr;
   rows.numAttrs = 2;
   for (int q = o->n_p - 1; q >= 0; --q) {
-    if ((e = launch_pdl(k_long_col_fwd, cols, col_threads, smem_col, s, la, q))) return e;
+    if ((e = launch_pdl(k_long_col_fwd, cols, dim3(col_threads), smem_col, s, la, q))) return e;
     if ((e = cudaLaunchKernelEx(&rows, k_long_rows, la))) return e;
-    if ((e = launch_pdl(k_long_col_inv, cols, col_threads, smem_col, s, la, q))) return e;
-    if ((e = launch_pdl(k_long_direct, dim3(152 * 4), dim3(256), 0, s, la, q))) return e;
+    if ((e = launch_pdl(k_long_col_inv, cols, dim3(col_threads), smem_col, s, la, q))) return e;
+    if ((e = launch_pdl(k_long_direct, dim3(DIRECT_CTAS), dim3(DIRECT_THREADS), smem_direct, s, la, q)))
+      return e;
   }
   return cudaGetLastError();
 }

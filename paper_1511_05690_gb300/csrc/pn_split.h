@@ -23,6 +23,20 @@ inline int image_split(int64_t xa, int64_t xb, int ctas) {
   return static_cast<int>(worst(hi) < worst(lo) ? hi : lo);
 }
 
+// Dynamic shared memory for the CTAs (of at most 64 registers a thread) of a kernel that is
+// bound per SM and that programmatic launch may place while the kernel before it
+// drains: `bytes`, or so much more that an SM holds no more of them than their even
+// share.  Otherwise the SMs that drain first take far more than the others (a
+// convolution of 50 and 300000 values over 5 levels: 1918 us, 1239 by plain launches,
+// whose empty levels cost 75 us in a call of one level).  More CTAs than fit at once
+// are placed as they end.
+constexpr int SM_SMEM = 228 * 1024, CTA_SMEM_MAX = 226 * 1024;  // (1 KB for static arrays)
+inline int even_share_smem(int bytes, int ctas, int threads, int sms) {
+  const int share = (ctas + sms - 1) / sms, fit = std::min(1024 / threads, 32);
+  if (share >= fit) return bytes;
+  return std::max(bytes, std::min(CTA_SMEM_MAX, (SM_SMEM / share - 1024) & ~1023));
+}
+
 // The affine fit's stream over B's rows (k_fit_stream): a thread per sample, the
 // samples' values of A for STREAM_K indices at a time, a ring of whole rows of B.
 constexpr int STREAM_THREADS = 1024;

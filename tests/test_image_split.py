@@ -22,6 +22,8 @@ def split(tmp_path_factory):
         'extern "C" int split(long long a, long long b, int n) { return pn::image_split(a, b, n); }\n'
         'extern "C" int ranges(long long N, long long K, long long f, int n_p, long long room) {\n'
         '  int stages = 0; return pn::fit_stream_ranges(N, K, f, n_p, room, 152, &stages); }\n'
+        'extern "C" int even(int bytes, int ctas, int threads, int sms) {\n'
+        '  return pn::even_share_smem(bytes, ctas, threads, sms); }\n'
         'static pn::DeviceSet set;\n'
         'extern "C" int add(int d) { int had = set.has(d); set.add(d); return had; }\n')
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "s.cpp"),
@@ -50,6 +52,24 @@ def test_the_affine_fit_streams_where_its_tests_mean_it_to(split):
     for N, K, f, room in ((4096, 4095, 1024, 1 << 30), (16388, 8192, 1024, 1 << 30),
                           (4096, 8192, 1024, 15 * 8 * 1024), (4096, 8192, 1025, 1 << 30)):
         assert ranges(N, K, f, 7, room) == 0
+
+
+def test_an_sm_holds_no_more_than_its_even_share(split):
+    even = ctypes.CDLL(split.lib).even
+    for threads in (32, 64, 128, 256, 512):
+        fit = min(1024 // threads, 32)
+        for ctas in (1, 151, 152, 153, 256, 304, 305, 512, 608, 1024, 2000):
+            for need in (0, 9000, 24576, 98304):
+                got, share = even(need, ctas, threads, 152), -(-ctas // 152)
+                assert need <= got <= 226 * 1024 or got == need
+                if share >= fit:
+                    assert got == need
+                    continue
+                held = (228 * 1024) // (got + 1024)  # 1 KB of each CTA is the system's
+                assert held <= share
+                if need <= (228 * 1024) // share - 2048:
+                    assert held * 152 >= ctas  # all still fit at once
+    assert even(24576, 512, 128, 0 + 152) == (228 * 1024 // 4 - 1024) // 1024 * 1024
 
 
 def _worst(xa, xb, n, ctas):
