@@ -1110,10 +1110,11 @@ int launch_images(const Common& cm, const Level& lv, void* stream, const Operand
   const bool ta = maps && maps->has_a && tma_fits(xa), tb = maps && maps->has_b && tma_fits(xb);
   int e = 0;
   if (ta && tb && tma_together(xa, xb)) return launch_tma(cm, lv, stream, *maps, xa, xb);
-  if (ta && xa > 0) e = launch_tma(cm, lv, stream, *maps, xa, 0);
-  if (!e && tb && xb > 0) e = launch_tma(cm, lv, stream, *maps, 0, xb);
-  const int pa = ta ? 0 : xa, pb = tb ? 0 : xb;
-  if (!e && pa + pb > 0) e = launch_power(cm, lv, stream, pa, pb);
+  // A's images first, then B's
+  if (!ta && !tb) return xa + xb > 0 ? launch_power(cm, lv, stream, xa, xb) : 0;
+  if (xa > 0) e = ta ? launch_tma(cm, lv, stream, *maps, xa, 0) : launch_power(cm, lv, stream, xa, 0);
+  if (!e && xb > 0)
+    e = tb ? launch_tma(cm, lv, stream, *maps, 0, xb) : launch_power(cm, lv, stream, 0, xb);
   return e;
 }
 
